@@ -122,8 +122,8 @@ merbit_status merbit_plan_get_info(merbit_plan_t plan, merbit_plan_info* info);
 merbit_status merbit_plan_export(merbit_plan_t plan, uint32_t* tile_x, uint32_t* tile_y,
                                  uint32_t* lane_desc, int32_t* block_row);
 
-/* Block kernels of the product y = A x (every call that multiplies by a plan's
- * matrix uses one of them; results agree to rounding):
+/* Kernels of the product y = A x (every call that multiplies by a plan's matrix uses
+ * one of them; results agree to rounding):
  *   MERBIT_KERNEL_CLASSIC: 256 threads per CTA; all of them gather x and form the
  *     products of a block, then each warp reduces one tile (Sec. 4.2, one block at
  *     a time per CTA, two copy stages).
@@ -135,9 +135,11 @@ merbit_status merbit_plan_export(merbit_plan_t plan, uint32_t* tile_x, uint32_t*
  *     the producers' work on block i + 1).
  *   A split kernel that cannot hold one CTA's stages on an SM (large sigma x block
  *   size with 8-byte values) gives way to CLASSIC.
- *   MERBIT_KERNEL_AUTO (the default): SPLIT while two of its CTAs fit on an SM and
- *     their three stages at the plan's sigma take at most 168 KB of shared memory per
- *     SM, else SPLIT2 while two of those fit, else CLASSIC. */
+ *   MERBIT_KERNEL_AUTO (the default): for sigma <= 14 without a hot-column table the
+ *     lane-walk kernel, in which every warp gathers, walks and commits its own tiles.
+ *     Otherwise SPLIT while two of its CTAs fit on an SM and their three stages at the
+ *     plan's sigma take at most 168 KB of shared memory per SM, else SPLIT2 while two
+ *     of those fit, else CLASSIC. */
 enum {
   MERBIT_KERNEL_AUTO = 0,
   MERBIT_KERNEL_CLASSIC = 1,

@@ -90,7 +90,9 @@ cudaError_t grow(void** buf, size_t* cap, size_t need) {
 
 cudaError_t reset_device_state(merbit_plan_s* p, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(p->red, 0, sizeof(RedState), st);
-  if (e == cudaSuccess && p->nb > 0) e = cudaMemsetAsync(p->bnd_acc, 0, sizeof(double) * (p->nb + 1), st);
+  // the tile accumulators follow the block accumulators
+  if (e == cudaSuccess && p->nb > 0)
+    e = cudaMemsetAsync(p->bnd_acc, 0, sizeof(double) * (size_t)(p->nb + 1 + p->tile_num + 1), st);
   return e;
 }
 
@@ -353,8 +355,14 @@ merbit_status merbit_plan_ex(const int32_t* row_ptr, const int32_t* col_idx, int
   if (e == cudaSuccess)
     e = cudaMalloc(&p->lane_desc, (size_t)p->desc_bytes * (size_t)std::max<int64_t>(p->lane_num, 1));
   if (e == cudaSuccess) e = cudaMalloc(&p->bnd_row, nbb);
-  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_slot, nbb);
-  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_acc, sizeof(double) * (size_t)(p->nb + 1));
+  // the tile slots and accumulators lie behind the block ones, in the same allocations
+  const size_t bounds = (size_t)(p->nb + 1) + (size_t)(p->tile_num + 1);
+  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_slot, sizeof(int32_t) * bounds);
+  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_acc, sizeof(double) * bounds);
+  if (e == cudaSuccess) {
+    p->tile_slot = p->bnd_slot + (p->nb + 1);
+    p->tile_acc = p->bnd_acc + (p->nb + 1);
+  }
   if (e == cudaSuccess) e = cudaMalloc(&p->part, sizeof(double2) * (size_t)kMaxParts);
   if (e == cudaSuccess) e = cudaMalloc(&p->red, sizeof(RedState));
   if (e == cudaSuccess) e = cudaMallocHost(&p->host_pinned, 256);

@@ -47,6 +47,8 @@ struct Geometry {
   const int32_t* bnd_row;
   const int32_t* bnd_slot;
   double* bnd_acc;
+  const int32_t* tile_slot;   // per tile: first tile that starts in the same row
+  double* tile_acc;           // per tile: FP64 accumulator of a row at a unit boundary
   double2* part;   // per-CTA reduction partials of the main kernel
   RedState* red;
   int n_rows;
@@ -54,6 +56,7 @@ struct Geometry {
   int steps;       // nnz + n_rows
   int sigma;
   int W;           // tiles per block
+  int unit;        // lane-walk kernel: consecutive tiles a warp takes at a time
   int stages;      // split kernel: stages in its ring (2 or 3)
   int desc64;      // lane descriptors are 64-bit words (sigma > 14)
   int fold;        // the block kernel's last CTA finishes the product (few blocks)
@@ -86,6 +89,8 @@ struct merbit_plan_s {
   int32_t* bnd_row = nullptr;
   int32_t* bnd_slot = nullptr;
   double* bnd_acc = nullptr;
+  int32_t* tile_slot = nullptr;          // tile_num + 1, behind bnd_slot; null: no lane-walk kernel
+  double* tile_acc = nullptr;            // tile_num + 1, behind bnd_acc
   double2* part = nullptr;               // kMaxParts entries
   merbit::RedState* red = nullptr;
   // lazily built PageRank data
@@ -108,6 +113,7 @@ struct merbit_plan_s {
     g.col_stage = col; g.hot_list = hot_list; g.hot_n = 0;   // a launch opts in to the table
     g.wait_limit = wait_limit;
     g.bnd_row = bnd_row; g.bnd_slot = bnd_slot;
+    g.tile_slot = tile_slot; g.tile_acc = tile_acc; g.unit = 1;
     g.bnd_acc = bnd_acc; g.part = part; g.red = red;
     g.n_rows = (int)n_rows; g.nnz = (int)nnz; g.steps = (int)(nnz + n_rows);
     g.sigma = sigma; g.W = tiles_per_block; g.stages = 3; g.desc64 = desc_bytes == 8; g.fold = 0;

@@ -80,26 +80,30 @@ __global__ void plan_tiles_kernel(const int32_t* __restrict__ row_ptr, int n_row
   }
 }
 
-// bnd_row[b] = ROW(tile_y[min(b*W, tile_num)]) for b = 0..nb.
-__global__ void plan_block_rows_kernel(const uint32_t* __restrict__ tile_y, int tile_num, int W,
-                                       int nb, int32_t* __restrict__ bnd_row) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b > nb) return;
-  bnd_row[b] = (int32_t)(tile_y[min(b * W, tile_num)] & ~kMsb);
-}
-
-// bnd_slot[b] = first index b' with bnd_row[b'] == bnd_row[b] (bnd_row is sorted).
-__global__ void plan_slots_kernel(const int32_t* __restrict__ bnd_row, int nb,
-                                  int32_t* __restrict__ bnd_slot) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b > nb) return;
-  const int key = bnd_row[b];
-  int lo = 0, hi = b;
+// Rows shared between tiles and between blocks.  For tile boundary i (row y of tile_y[i]):
+// tile_slot[i] = first boundary in the same row (the rows are non-decreasing).  Block
+// boundary b is tile boundary min(b*W, tile_num): bnd_row[b] its row, bnd_slot[b] the first
+// block boundary in that row, which is the first one at or after the tile slot.
+__global__ void plan_bounds_kernel(const uint32_t* __restrict__ tile_y, int tile_num, int W, int nb,
+                                   int32_t* __restrict__ tile_slot, int32_t* __restrict__ bnd_row,
+                                   int32_t* __restrict__ bnd_slot) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i > tile_num) return;
+  const bool block = i % W == 0 || i == tile_num;
+  if (!tile_slot && !block) return;
+  const int key = (int)(__ldg(tile_y + i) & ~kMsb);
+  int lo = 0, hi = i;
+  if (i > 0 && (int)(__ldg(tile_y + i - 1) & ~kMsb) < key) lo = i;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (bnd_row[mid] < key) lo = mid + 1; else hi = mid;
+    if ((int)(__ldg(tile_y + mid) & ~kMsb) < key) lo = mid + 1; else hi = mid;
   }
-  bnd_slot[b] = lo;
+  if (tile_slot) tile_slot[i] = lo;
+  if (block) {
+    const int b = i == tile_num ? nb : i / W;
+    bnd_row[b] = key;
+    bnd_slot[b] = (lo + W - 1) / W;
+  }
 }
 
 __global__ void mark_columns_kernel(const int32_t* __restrict__ col, int nnz,
@@ -138,10 +142,9 @@ cudaError_t build_tiles(const merbit_plan_s* p, const int32_t* row_ptr, cudaStre
         p->tile_y, p->lane_desc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int nbt = (int)((p->nb + 1 + threads - 1) / threads);
-  plan_block_rows_kernel<<<nbt, threads, 0, st>>>(p->tile_y, (int)p->tile_num, p->tiles_per_block,
-                                                  (int)p->nb, p->bnd_row);
-  plan_slots_kernel<<<nbt, threads, 0, st>>>(p->bnd_row, (int)p->nb, p->bnd_slot);
+  const int nbt = (int)((p->tile_num + 1 + threads - 1) / threads);
+  plan_bounds_kernel<<<nbt, threads, 0, st>>>(p->tile_y, (int)p->tile_num, p->tiles_per_block, (int)p->nb,
+                                              p->tile_slot, p->bnd_row, p->bnd_slot);
   return cudaGetLastError();
 }
 

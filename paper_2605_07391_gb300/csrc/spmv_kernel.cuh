@@ -8,6 +8,8 @@
 //     two cp.async.bulk copies completing on an mbarrier, issued ahead of use
 //     (the block's nonzero range is contiguous, so one bulk copy per array
 //     suffices);
+//   * the automatic choice for sigma <= 14 is the lane-walk kernel of
+//     spmv_walk_kernel.cuh, whose warps work alone;
 //   * two block kernels share the stages and the per-tile reduction:
 //     merbit_spmv_kernel (all threads gather, then all reduce; two stages) and
 //     merbit_spmv_split_kernel (producer threads gather for the next blocks
@@ -1103,6 +1105,10 @@ inline size_t add_hot_table(const merbit_plan_s* p, Geometry& g, const void* ker
   return need;
 }
 
+}  // namespace merbit
+#include "spmv_walk_kernel.cuh"
+namespace merbit {
+
 // Grid, dynamic shared memory and geometry (with or without the hot-column table) of the
 // split kernel's launch for a plan; false if two of its CTAs do not fit on an SM (or
 // none does, when `forced`).
@@ -1137,7 +1143,8 @@ template <typename VT, typename XT, typename AT, typename Epi>
 cudaError_t launch_spmv(const merbit_plan_s* p, const VT* vals, const XT* x, const Epi& epi,
                         cudaStream_t st) {
   if (p->nb == 0) return cudaSuccess;
-  // The split kernel is the default while two of its CTAs fit on an SM (measured on
+  // The lane-walk kernel is the automatic choice where it applies.  Otherwise (sigma > 14, a
+  // hot-column table, no tile slots) the split kernel is the default while two of its CTAs fit on an SM (measured on
   // sm_103a, R-MAT scale 21 and 24: 15-30 % faster than the classic kernel for 32- and
   // 64-bit values, 11 % for 16-bit values at sigma 14, slower with one CTA per SM).
   Geometry g = p->geom();
@@ -1146,6 +1153,7 @@ cudaError_t launch_spmv(const merbit_plan_s* p, const VT* vals, const XT* x, con
   int grid = 0;
   bool split = false;
   const int kind = p->spmv_kernel;
+  if (kind == MERBIT_KERNEL_AUTO && walk_takes(p)) return launch_walk<VT, XT, AT, Epi>(p, vals, x, epi, st);
   // A split kernel that was asked for but cannot hold even one CTA's stages on an SM (large
   // sigma x block size with 8-byte values) gives way to the classic kernel, whose ring
   // has two stages.
