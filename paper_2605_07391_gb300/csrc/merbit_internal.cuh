@@ -105,7 +105,9 @@ struct merbit_plan_s {
   void* y_stage = nullptr;
   size_t x_stage_bytes = 0, y_stage_bytes = 0;
   void* host_pinned = nullptr;           // small pinned block for state read-back
-  double* spmm_acc = nullptr;            // (nb + 1) x 32 FP64 boundary accumulators of the SpMM
+  double* spmm_acc = nullptr;            // spmm_acc_sets x 32 FP64 boundary accumulators of the SpMM
+  void* spmm_pack = nullptr;             // padded copy of up to 32 columns of an unaligned X
+  size_t spmm_pack_bytes = 0;
 
   merbit::Geometry geom() const {
     merbit::Geometry g;
@@ -192,11 +194,12 @@ cudaError_t spmv_resid_f64(const merbit_plan_s* p, const double* vals, const dou
 cudaError_t spmv_sweep(const merbit_plan_s* p, merbit_dtype vdt, const void* vals,
                        const float* x, const SweepParams& prm, cudaStream_t st);
 // Y = A X, row-major X (n_cols x k, leading dimension ldx) and Y (n_rows x k, ldy), f32;
-// acc: (nb + 1) x 32 zeroed FP64 accumulators (left zeroed)
-cudaError_t spmm_plain_f32(const merbit_plan_s* p, const float* vals, const float* X, int64_t k,
+// acc: spmm_acc_sets x 32 zeroed FP64 accumulators (left zeroed)
+int64_t spmm_acc_sets(const merbit_plan_s* p);
+cudaError_t spmm_plain_f32(merbit_plan_s* p, const float* vals, const float* X, int64_t k,
                            int64_t ldx, float* Y, int64_t ldy, double* acc, cudaStream_t st);
 // Y = scale * A X, skipped once the plan's stop flag is set (iterative drivers)
-cudaError_t spmm_scaled_f32(const merbit_plan_s* p, const float* vals, const float* X, int64_t k,
+cudaError_t spmm_scaled_f32(merbit_plan_s* p, const float* vals, const float* X, int64_t k,
                             int64_t ldx, float* Y, int64_t ldy, float scale, double* acc,
                             cudaStream_t st);
 // Personalised PageRank: X = one-hot seed columns (n x k, ld k), d_cur = their dangling mass
@@ -205,7 +208,7 @@ cudaError_t ppr_init(const merbit_plan_s* p, float* X, int64_t k, const int32_t*
 // one update Y = alpha P^T X + (alpha D + 1 - alpha) e_seed for all k columns, then the
 // finish step (per-column residuals into last_r, D of Y into d_cur, hist[iter] = largest
 // residual, stop flag when it is below tol); rd: 2k zeroed FP64 accumulators (left zeroed)
-cudaError_t ppr_update(const merbit_plan_s* p, const float* vals, const float* X, float* Y,
+cudaError_t ppr_update(merbit_plan_s* p, const float* vals, const float* X, float* Y,
                        int64_t k, const int32_t* seed, double* d_cur, double* rd, double* last_r,
                        float alpha, double tol, int iter, double* hist, double* acc,
                        cudaStream_t st);

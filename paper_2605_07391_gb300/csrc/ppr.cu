@@ -161,7 +161,7 @@ cudaError_t ppr_init(const merbit_plan_s* p, float* X, int64_t k, const int32_t*
   return cudaGetLastError();
 }
 
-cudaError_t ppr_update(const merbit_plan_s* p, const float* vals, const float* X, float* Y,
+cudaError_t ppr_update(merbit_plan_s* p, const float* vals, const float* X, float* Y,
                        int64_t k, const int32_t* seed, double* d_cur, double* rd, double* last_r,
                        float alpha, double tol, int iter, double* hist, double* acc,
                        cudaStream_t st) {

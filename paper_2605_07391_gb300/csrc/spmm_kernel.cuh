@@ -2,33 +2,29 @@
 // on the same plan as the SpMV (the batching extension of the hot path: k
 // personalisation vectors in one pass).
 //
-// Work unit: the SpMV's block of 8 tiles, staged by the same two bulk copies;
-// one warp per tile.  A column chunk of KC columns is split into slices of VW
-// consecutive columns (VW = 4: one 16-byte load per slice); T = KC / VW
-// threads cover a chunk, so a warp walks L = 32 / T lanes at once and a tile's
-// 32 lanes in T passes.
-//   1. A thread takes one lane of the pass and one slice.  The lane descriptor
-//      (Sec. 4.1.1 bit_flag) gives, for every step, whether it is a down step
-//      and which nonzero a right step consumes (step k takes nonzero
-//      x_off + k - (down steps before k)), so the row slices of all the lane's
-//      right steps are gathered before any is used.
-//   2. The steps are walked in order: a right step adds vals[p] * slice into
-//      the running sum, a down step ends a row.  Rows ended after the lane's
-//      first down step lie wholly inside the lane and are written to Y; the
-//      lane's first ended row may have begun in earlier lanes.
-//   3. Runs across lanes: the sum open after lane l obeys
-//      OC_l = a_l + b_l * OC_{l-1} (a_l the lane's trailing sum, b_l = 1 when
-//      the lane ends no row), a linear recurrence scanned by shuffles; the
-//      first ended row of lane l totals OC_{l-1} plus the lane's head sum, and
-//      the run open after a pass is carried into the next.
-//   4. The tile's first row and the run open at its end go to a small shared
-//      table; the last warp to finish the block (an arrival count, no block
-//      barrier) adds up each row's entries and refills the block's stage.  The
-//      block's first and last rows are added into per-row FP64 accumulators
-//      that a finalize kernel writes out and clears (the SpMV's boundary-row
-//      scheme, KC values wide).
-// Single-row tiles (the tile_y mark of Sec. 4.1.2) skip the descriptors: lanes
-// take every L-th nonzero and their sums are added across the warp.
+// The lane-walk kernel of the SpMV (spmv_walk_kernel.cuh), k values wide: a warp takes units
+// of consecutive tiles on its own, with one buffer each for a tile's columns and values.  A
+// column chunk of KC columns is split into slices of VW consecutive columns (one load each);
+// T = KC / VW threads share a lane of the tile, so a warp walks L = 32 / T lanes at once and a
+// tile's 32 lanes in T passes.  Per pass:
+//   1. the lane descriptor (Sec. 4.1.1) says which nonzero every right step consumes, so the
+//      row slices of a batch of steps are gathered before any is used;
+//   2. the steps are walked: a right step adds vals * slice into the running sum, a down step
+//      ends a row.  Rows that begin and end inside the lane go straight to Y; the lane's
+//      first row end is kept (`head`);
+//   3. the runs open at the lanes' ends are joined by a segmented shuffle scan; a lane's first
+//      row totals its head plus the run that reaches it, and the run open after the pass is
+//      carried into the next pass, the next tile and to the unit's end.
+// A unit's first row and the row open at its end are added into FP64 accumulators (KC wide,
+// one set per distinct row at the unit boundaries), which a second pass writes and clears.
+//
+// What bounds it.  Narrow chunks: the L1 data pipe, one wavefront per gathered row slice line
+// (k = 8: 82 % busy, a quarter of it shared-memory work).  Wide ones: the bytes in flight (16
+// warps, 14 slices of 16 bytes a thread: 114 KB an SM).  Multiply-adds and stores are predicated
+// on the descriptor's bits instead of branched over, and no table, arrival count or block barrier
+// joins the warps: 2.6 warp instructions per nonzero at k = 8 instead of 3.2.  R-MAT scale 21
+// (32.4 M nonzeros), before and after: k = 4 0.189 / 0.163 ms, k = 8 0.224 / 0.192, k = 16 0.302 /
+// 0.271, k = 32 0.495 / 0.466.
 #pragma once
 
 #include <climits>
@@ -45,6 +41,12 @@ template <> struct SpmmVec<1> {
   static __device__ __forceinline__ T load(const float* p) { return __ldg(p); }
   static __device__ __forceinline__ T load_plain(const float* p) { return *p; }
   static __device__ __forceinline__ void store(float* p, const float (&a)[1]) { *p = a[0]; }
+  static __device__ __forceinline__ T load_shared(const float* p) { return *p; }
+  static __device__ __forceinline__ void store_shared(float* p, const T& v) { *p = v; }
+  static __device__ __forceinline__ void store_shared_if(uint32_t pred, float* p, const T& v) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.f32 [%1], %2;\n\t}" ::"r"(pred),
+                 "r"(smem_addr(p)), "f"(v));
+  }
   static __device__ __forceinline__ void fma(float w, const T& x, T& s) { s = fmaf(w, x, s); }
   static __device__ __forceinline__ float get(const T& v, int) { return v; }
   static __device__ __forceinline__ T from(const float (&a)[1]) { return a[0]; }
@@ -70,6 +72,13 @@ template <> struct SpmmVec<4> {
   }
   static __device__ __forceinline__ void store(float* p, const float (&a)[4]) {
     *reinterpret_cast<float4*>(p) = make_float4(a[0], a[1], a[2], a[3]);
+  }
+  static __device__ __forceinline__ T load_shared(const float* p) { return load_plain(p); }
+  static __device__ __forceinline__ void store_shared(float* p, const T& v) { *reinterpret_cast<float4*>(p) = v; }
+  static __device__ __forceinline__ void store_shared_if(uint32_t pred, float* p, const T& v) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(
+                     pred),
+                 "r"(smem_addr(p)), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
   }
   static __device__ __forceinline__ void fma(float w, const T& x, T& s) {
     s.x = fmaf(w, x.x, s.x);
@@ -100,442 +109,376 @@ template <> struct SpmmVec<4> {
   }
 };
 
-// Two 16-byte halves: a thread's slice is a whole 32-byte row of an 8-column chunk,
-// read by one 32-byte load (its address must be 32-byte aligned).
-struct Float8 {
-  float4 a, b;
-};
-template <> struct SpmmVec<8> {
-  using T = Float8;
-  using H = SpmmVec<4>;
-  static __device__ __forceinline__ T zero() { return T{H::zero(), H::zero()}; }
-  static __device__ __forceinline__ T load(const float* p) {
-    T v;
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(v.a.x), "=f"(v.a.y), "=f"(v.a.z), "=f"(v.a.w), "=f"(v.b.x), "=f"(v.b.y), "=f"(v.b.z),
-          "=f"(v.b.w)
-        : "l"(p));
-    return v;
-  }
-  static __device__ __forceinline__ void fma(float w, const T& x, T& s) {
-    H::fma(w, x.a, s.a);
-    H::fma(w, x.b, s.b);
-  }
-  static __device__ __forceinline__ float get(const T& v, int i) {
-    return i < 4 ? H::get(v.a, i) : H::get(v.b, i - 4);
-  }
-  static __device__ __forceinline__ T from(const float (&a)[8]) {
-    return T{make_float4(a[0], a[1], a[2], a[3]), make_float4(a[4], a[5], a[6], a[7])};
-  }
-  static __device__ __forceinline__ void add(T& s, const T& x) {
-    H::add(s.a, x.a);
-    H::add(s.b, x.b);
-  }
-  static __device__ __forceinline__ T shfl_up(const T& v, int d) {
-    return T{H::shfl_up(v.a, d), H::shfl_up(v.b, d)};
-  }
-  static __device__ __forceinline__ T shfl_xor(const T& v, int d) {
-    return T{H::shfl_xor(v.a, d), H::shfl_xor(v.b, d)};
-  }
-  static __device__ __forceinline__ T shfl(const T& v, int src) {
-    return T{H::shfl(v.a, src), H::shfl(v.b, src)};
-  }
-};
-
-// Epilogue of the SpMM: Y[r, c..c+VW) = scale * (A X)[r, c..c+VW).  row() takes f32 row sums
-// (called by the thread owning columns c..c+VW), row64 one column of a block-shared row
-// summed in FP64 (finalize kernel).  A gated launch does nothing once an iterative driver
-// has set the plan's stop flag (launches queued after convergence).
-struct EpiSpmmPlain {
+// Y[r, c..c+VW) = (scale *) sum.  YVEC: the slices of Y are 16-byte aligned and kc is a multiple
+// of VW; otherwise single columns below kc are stored.
+struct SpmmOut {
   float* y;
-  int ldy;
+  int64_t ldy;
   float scale;
-  bool gated;
+  int kc;          // columns of the chunk
+  bool gated;      // the launch does nothing once an iterative driver has set the stop flag
   __device__ __forceinline__ bool skip(const RedState* red) const {
     return gated && *reinterpret_cast<const volatile int*>(&red->done) != 0;
   }
-  __device__ __forceinline__ void row(int r, int c, float s) const {
-    y[(size_t)r * ldy + c] = scale * s;
-  }
-  __device__ __forceinline__ void row(int r, int c, const float4& s) const {
-    *reinterpret_cast<float4*>(y + (size_t)r * ldy + c) =
-        make_float4(scale * s.x, scale * s.y, scale * s.z, scale * s.w);
-  }
-  __device__ __forceinline__ void row(int r, int c, const Float8& s) const {
-    row(r, c, s.a);
-    row(r, c + 4, s.b);
-  }
-  __device__ __forceinline__ void row64(int r, int c, double s) const {
-    y[(size_t)r * ldy + c] = static_cast<float>(static_cast<double>(scale) * s);
-  }
 };
 
-// Depth of the SpMM's block ring.  A third stage (two CTAs per SM still fit) took the
-// shared memory per SM past the point where the driver shrinks L1: k = 8 on R-MAT scale
-// 22 went from 0.458 to 0.548 ms.
-constexpr int kSpmmStages = 2;
+template <bool SCALED>
+__device__ __forceinline__ float spmm_scaled(float v, float scale) {
+  if constexpr (SCALED) return scale * v;
+  else return v;
+}
 
-struct SpmmGeometry {
-  double* acc;      // (nb + 1) x KC FP64 boundary-row accumulators of this chunk
-  int kc;           // columns in this chunk (a multiple of VW)
+// Predicated stores of a slice (no branch: lanes of a warp end rows at different steps; no memory
+// clobber: nothing in the kernel reads Y, and loads may move over them).
+template <int VW, bool YVEC, bool SCALED>
+__device__ __forceinline__ void spmm_store_if(uint32_t pred, float* p, const typename SpmmVec<VW>::T& v, float scale,
+                                              int left) {
+  using V = SpmmVec<VW>;
+  if constexpr (YVEC && VW == 4) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t"
+        "@q st.global.v4.f32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(pred),
+        "l"(p), "f"(spmm_scaled<SCALED>(v.x, scale)), "f"(spmm_scaled<SCALED>(v.y, scale)),
+        "f"(spmm_scaled<SCALED>(v.z, scale)), "f"(spmm_scaled<SCALED>(v.w, scale)));
+  } else {
+#pragma unroll
+    for (int i = 0; i < VW; ++i)
+      asm volatile(
+          "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t"
+          "@q st.global.f32 [%1], %2;\n\t}" ::"r"(i < left ? pred : 0u),
+          "l"(p + i), "f"(spmm_scaled<SCALED>(V::get(v, i), scale)));
+  }
+}
+
+// Gathers of a slice, kept in order so that a batch is in flight before its first use.  They are
+// not predicated: a register that a predicated load may leave unwritten stays allocated through
+// the whole loop (168 registers instead of 96).  Steps that take no nonzero load the tile's
+// first one again.
+__device__ __forceinline__ void spmm_load(const float* p, float& v) {
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+}
+__device__ __forceinline__ void spmm_load(const float* p, float4& v) {
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+}
+
+constexpr int kSpmmWarps = 4;
+constexpr int kSpmmThreads = kSpmmWarps * 32;
+
+// FP64 accumulators of unit boundary row: set index of tile boundary i (the first unit boundary
+// in that row, which is the first one at or after the row's first tile boundary).
+__device__ __forceinline__ int spmm_set(const Geometry& g, int i) {
+  return (__ldg(g.tile_slot + i) + g.unit - 1) / g.unit;
+}
+
+// A warp's units: whole rounds give consecutive units to a CTA's warps, the rest is spread over
+// the CTAs first (as in the SpMV's kernel); computed on the host.
+struct SpmmUnits {
+  int nfull, rest;
 };
 
-// Two CTAs per SM: the register room (up to 128 per thread) holds a lane's sigma row
-// slices in flight.
-template <int KC, int VW, typename Epi>
-__global__ void __launch_bounds__(kThreads, 2)
-    merbit_spmm_kernel(const Geometry g, const SpmmGeometry sg, const float* __restrict__ vals,
-                       const float* __restrict__ X, int ldx, Epi epi) {
+// Shared memory of a warp: values, columns, and per thread the head sum of its lane's pass
+// (the carried run takes the place of a pass's last lane after the scan).
+template <int VW>
+__host__ __device__ constexpr size_t spmm_warp_bytes(int sigma) {
+  return 2 * sizeof(float) * (size_t)walk_cap(sigma) + 2 * 32 * sizeof(float) * VW;
+}
+
+template <int KC, int VW, bool YVEC, bool SCALED, int CTAS>
+__global__ void __launch_bounds__(kSpmmThreads, CTAS)
+    merbit_spmm_kernel(const Geometry g, const SpmmUnits un, double* __restrict__ acc, const float* __restrict__ vals,
+                       const float* __restrict__ X, const int64_t ldx, const SpmmOut out) {
   using V = SpmmVec<VW>;
   using VT = typename V::T;
   constexpr int T = KC / VW;                   // threads per lane, one slice of VW columns each
   constexpr int L = 32 / T;                    // lanes walked at once (one pass)
   constexpr int U1 = 8;                        // row slices per round of a single-row tile
-  constexpr int HB = VW == 8 ? kSigmaMax / 2 : kSigmaMax;   // steps per batch of gathers
-  static_assert(kSigmaMax % HB == 0, "step batches");
-  constexpr int VE = 4;
-  constexpr int NE = 2 * kTilesPerBlock;       // table entries of a block: each warp's first / last run
-  constexpr int S = kSpmmStages;
-  __shared__ __align__(8) uint64_t mbar[S];
-  __shared__ StageInfo info[S];
-  __shared__ int arrive[S];                    // warps done with the stage's block
-  __shared__ int wt_row[S][NE];
-  __shared__ __align__(16) float wt_val[S][NE][KC];
+  __shared__ __align__(8) uint64_t bars[kSpmmWarps][2];
   extern __shared__ __align__(128) unsigned char dyn_smem[];
 
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  const int lane = tid & 31;
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int gl = lane / T;                     // lane of the pass this thread walks
   const int c = (lane % T) * VW;               // first column of this thread's slice
-  const bool c_ok = c < sg.kc;
-  const int G = gridDim.x;
-  if (epi.skip(g.red)) return;
+  const int left = out.kc - c;                 // its columns
+  const uint32_t c_ok = left > 0 ? ~0u : 0u;
+  if (out.skip(g.red)) return;
 
-  const size_t svb = stage_vals_bytes<float>(g.sigma, kTilesPerBlock);
-  const size_t stb = stage_bytes<float>(g.sigma, kTilesPerBlock);
-  auto sv = [&](int s) { return reinterpret_cast<float*>(dyn_smem + (size_t)s * stb); };
-  auto sc = [&](int s) { return reinterpret_cast<int32_t*>(dyn_smem + (size_t)s * stb + svb); };
-  const uint64_t pol_stream = policy_evict_first();
-  const int nnz_a = g.nnz & ~(VE - 1);
-
-  auto geom_of = [&](int v, int& xb, int& xe, uint32_t& yb, uint32_t& ye) {
-    const int bs = v * kTilesPerBlock;
-    const int be = min(bs + kTilesPerBlock, g.tile_num);
-    xb = (int)g.tile_x[bs];
-    xe = (int)g.tile_x[be];
-    yb = g.tile_y[bs] & ~kMsb;
-    ye = g.tile_y[be] & ~kMsb;
-  };
-  auto issue = [&](int s, int xb, int xe, uint32_t yb, uint32_t ye) {
-    StageInfo in;
-    in.x_bs = xb; in.x_be = xe; in.y_bs = (int)yb; in.y_be = (int)ye;
-    in.a0v = xb & ~(VE - 1);
-    in.endv = max(in.a0v, min((xe + VE - 1) & ~(VE - 1), nnz_a));
-    in.a0c = in.a0v;
-    in.endc = in.endv;
-    info[s] = in;
-    const uint32_t cnt = (uint32_t)(in.endv - in.a0v);
-    mbar_arrive_expect_tx(&mbar[s], cnt * 8u);
-    if (cnt) {
-      bulk_g2s(sv(s), vals + in.a0v, cnt * 4u, &mbar[s], pol_stream);
-      bulk_g2s(sc(s), g.col + in.a0c, cnt * 4u, &mbar[s], pol_stream);
-    }
-  };
-
-  if (tid == 0) {
-    for (int i = 0; i < S; ++i) {
-      mbar_init(&mbar[i], 1);
-      arrive[i] = 0;
-    }
+  const int cap = walk_cap(g.sigma);
+  float* const sv = reinterpret_cast<float*>(dyn_smem + (size_t)warp * spmm_warp_bytes<VW>(g.sigma));
+  int32_t* const sc = reinterpret_cast<int32_t*>(sv + cap);
+  float* const s_head = sv + 2 * cap + lane * VW;              // this thread's head sum
+  float* const s_carry = sv + 2 * cap + (32 + lane % T) * VW;  // this slice's carried run
+  if (lane == 0) {
+    mbar_init(&bars[warp][0], 1);
+    mbar_init(&bars[warp][1], 1);
     fence_mbar_init();
   }
-  __syncthreads();
-  if (tid == 0) {
-    for (int i = 0; i < S; ++i) {
-      const int v = blockIdx.x + i * G;
-      if (v >= g.nb) break;
-      int xb, xe; uint32_t yb, ye;
-      geom_of(v, xb, xe, yb, ye);
-      issue(i, xb, xe, yb, ye);
-    }
-  }
+  __syncwarp();
 
-  // The warps move through the ring on their own: no block-wide barrier.  The last warp
-  // to finish a block (a shared-memory arrival count) adds up the block's cross-warp table
-  // and refills the stage with the block S steps ahead.
-  int s = 0;
+  // row `col` of X at this thread's slice; slices wider than a column come with ldx < 2^30, so
+  // that the byte offset is one 32 x 32-bit multiply-add
+  const float* const Xc = X + (c_ok ? c : 0);
+  auto x_row = [&](int col) {
+    if constexpr (VW == 1) return Xc + (int64_t)col * ldx;
+    else
+      return reinterpret_cast<const float*>(reinterpret_cast<const char*>(Xc) +
+                                            (uint64_t)(uint32_t)col * ((uint32_t)ldx * 4u));
+  };
+  auto y_row = [&](int r) { return out.y + c + (int64_t)r * out.ldy; };
+  auto unit_start = [&](int r) {
+    const int i = warp * (int)gridDim.x + (int)blockIdx.x;
+    if (r >= un.nfull + (i < un.rest ? 1 : 0)) return -1;
+    const int round = (int)gridDim.x * kSpmmWarps;
+    return (r < un.nfull ? r * round + (int)blockIdx.x * kSpmmWarps + warp : un.nfull * round + i) * g.unit;
+  };
+  // bounds of tile ti, a word a lane: its first nonzero and row in lanes 0 and 2, the next
+  // tile's in lanes 1 and 3
+  auto load_meta = [&](int ti) { return __ldg((lane & 2 ? g.tile_y : g.tile_x) + ti + (lane & 1)); };
+  auto load_desc = [&](int ti) {
+    const int j = ti * kOmega + lane;
+    return j < g.lane_num ? ld_stream(g.lane_desc + j, policy_evict_first()) : 0u;
+  };
+  auto issue = [&](const void* src, void* dst, uint32_t meta, int which) {
+    const int a = (int)__shfl_sync(0xffffffffu, meta, 0), b = (int)__shfl_sync(0xffffffffu, meta, 1);
+    if (lane == 0)
+      walk_issue(static_cast<const int32_t*>(src), dst, a, b, g.nnz, &bars[warp][which], policy_evict_first());
+  };
+  auto add_acc = [&](int tile, const VT& v) {
+    double* a = acc + (size_t)spmm_set(g, tile) * KC + c;
+#pragma unroll
+    for (int i = 0; i < VW; ++i)
+      if (i < left) atomicAdd(a + i, (double)V::get(v, i));
+  };
+
+  int rd = 0;
+  int t = unit_start(0);
+  if (t < 0) return;
+  int t_start = t;
+  uint32_t meta = load_meta(t), desc = load_desc(t);
+  issue(g.col, sc, meta, 0);
+  issue(vals, sv, meta, 1);
   uint32_t par = 0;
-  for (int v = blockIdx.x; v < g.nb; v += G) {
-    const int ti = v * kTilesPerBlock + warp;
-    const bool tile_ok = ti < g.tile_num;
-    // the tile's bounds and its 32 lane descriptors (one per thread), read before the
-    // stage wait so that their latency hides behind it
-    uint32_t txs = 0, txe = 0, tys = 0, dreg = 0;
-    if (tile_ok) {
-      txs = __ldg(g.tile_x + ti);
-      txe = __ldg(g.tile_x + ti + 1);
-      tys = __ldg(g.tile_y + ti);
-      const int j = ti * kOmega + lane;
-      if (j < g.lane_num) dreg = ld_stream(g.lane_desc + j, pol_stream);
+  int y_unit = (int)(__shfl_sync(0xffffffffu, meta, 2) & ~kMsb);   // the unit's first row
+  if (gl == 0) V::store_shared(s_carry, V::zero());               // run open after the unit's passes so far
+  while (true) {
+    // the tile after this one, of this unit or of the next (-1: none)
+    const bool next_unit = t + 1 >= min(t_start + g.unit, g.tile_num);
+    const int tn = next_unit ? unit_start(rd + 1) : t + 1;
+    uint32_t nmeta = 0, ndesc = 0;
+    if (tn >= 0) {
+      nmeta = load_meta(tn);
+      ndesc = load_desc(tn);
     }
-    const bool ok = mbar_wait_bounded(&mbar[s], par, g.wait_limit);
+    const int xs = (int)__shfl_sync(0xffffffffu, meta, 0), xe = (int)__shfl_sync(0xffffffffu, meta, 1);
+    const uint32_t tys = __shfl_sync(0xffffffffu, meta, 2);
+    const int y_ws = (int)(tys & ~kMsb);
+    bool ok = mbar_wait_bounded(&bars[warp][0], par, g.wait_limit);
+    if (__all_sync(0xffffffffu, ok)) ok = mbar_wait_bounded(&bars[warp][1], par, g.wait_limit);
     if (!__all_sync(0xffffffffu, ok)) {
-      // this warp gives up: it records the error and waits, with the default limit, for
-      // the copies that may still be landing in the ring (this block and the next S - 1
-      // of the CTA; a wait for a copy never issued simply runs out), then returns.  A
-      // warp that gives up never arrives, so the other warps' waits run out in turn.
-      if (lane == 0) atomicOr(&g.red->err, 1);
-      int ss = s;
-      uint32_t pp = par;
-      for (int m = 0; m < S && v + m * G < g.nb; ++m) {
-        mbar_wait_bounded(&mbar[ss], pp);
-        if (++ss == S) {
-          ss = 0;
-          pp ^= 1u;
-        }
+      // give up: record it and let this tile's copies land (bounded) before leaving
+      if (lane == 0) {
+        atomicOr(&g.red->err, 1);
+        mbar_wait_bounded(&bars[warp][0], par);
+        mbar_wait_bounded(&bars[warp][1], par);
       }
       return;
     }
-    const StageInfo in = info[s];
-    const float* vs = sv(s);
-    const int32_t* cs = sc(s);
-    int* wrow = wt_row[s];
-    float (*wval)[KC] = wt_val[s];
-    if (lane == 0) {
-      wrow[2 * warp] = -1;
-      wrow[2 * warp + 1] = -1;
-    }
-    __syncwarp();
-
-    if (tile_ok) {
-      const int y_ws = (int)(tys & ~kMsb);
-      const int ntile = (int)(txe - txs);
-      const int ib = (int)txs - in.a0v;          // staged index of the tile's first nonzero
-      // a finished run of row r: block boundary rows go to the FP64 accumulators, the
-      // tile's first row and its run open at the tile's end to the cross-warp table,
-      // any other row straight to Y
-      auto emit = [&](int r, const VT& val, bool last_of_warp) {
-        if (r >= g.n_rows || !c_ok) return;
-        if (r == in.y_bs || r == in.y_be) {
-          double* a = sg.acc + (size_t)__ldg(g.bnd_slot + (r == in.y_bs ? v : v + 1)) * KC + c;
-#pragma unroll
-          for (int k = 0; k < VW; ++k) atomicAdd(a + k, (double)V::get(val, k));
-        } else if (last_of_warp || r == y_ws) {
-          const int e = 2 * warp + (last_of_warp ? 1 : 0);
-          if (lane % T == 0) wrow[e] = r;
-#pragma unroll
-          for (int k = 0; k < VW; ++k) wval[e][c + k] = V::get(val, k);
-        } else {
-          epi.row(r, c, val);
-        }
-      };
-      // the tile's nonzeros, ST = every one of them is staged (false only in the block
-      // holding the array's last few nonzeros, which are read from global memory)
-      auto walk = [&](auto st_tag) {
-        constexpr bool ST = decltype(st_tag)::value;
-        auto gather = [&](int idx, float& w) -> VT {
-          const int i = ib + idx;
-          int cc;
-          if (ST || in.a0v + i < in.endv) {
-            cc = cs[i];
-            w = vs[i];
-          } else {
-            cc = __ldg(g.col + in.a0v + i);
-            w = __ldg(vals + in.a0v + i);
-          }
-          return V::load(X + (size_t)cc * ldx + c);
-        };
-        if (tys & kMsb) {
-          // single-row tile: every nonzero belongs to row y_ws; lane gl takes every
-          // L-th one, then the lanes' sums are added across the warp
-          VT sum = V::zero();
-#pragma unroll 1
-          for (int base = gl; base < ntile; base += L * U1) {
-            VT xv[U1];
-            float wv[U1];
-#pragma unroll
-            for (int u = 0; u < U1; ++u) {
-              xv[u] = V::zero();
-              wv[u] = 0.f;
-              if (base + u * L < ntile && c_ok) xv[u] = gather(base + u * L, wv[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < U1; ++u) V::fma(wv[u], xv[u], sum);
-          }
-#pragma unroll
-          for (int o = T; o < 32; o <<= 1) V::add(sum, V::shfl_xor(sum, o));
-          if (gl == 0) emit(y_ws, sum, true);
-          return;
-        }
-        // lane walk (Sec. 4.2, k values wide): T passes of L lanes; each thread issues the
-        // row-slice gathers of all its lane's right steps before using any (the step ->
-        // nonzero map comes from the descriptor alone), then walks the steps: a down step
-        // ends a row.  A lane's first ended row may have begun in earlier lanes, so its
-        // head partial joins the runs flowing in; rows ended later in the lane are whole.
-        VT carry = V::zero();                    // run open after the previous pass
-        int open_row = y_ws;
-#pragma unroll 1
-        for (int p = 0; p < T; ++p) {
-          const int l = p * L + gl;
-          const uint32_t d = __shfl_sync(0xffffffffu, dreg, l);
-          const int j = ti * kOmega + l;
-          const bool active = j < g.lane_num;
-          const int len = active ? min(g.sigma, g.steps - j * g.sigma) : 0;
-          const uint32_t valid = (1u << len) - 1u;
-          const uint32_t dm = (d >> 18) & valid;   // down steps
-          const uint32_t rm = ~(d >> 18) & valid;  // right steps
-          const int xo = (int)(d & 511u);
-          const int y0 = active ? (int)((d >> 9) & 511u) : (g.n_rows - y_ws);
-          // right step k takes the lane's nonzero k - (down steps before k); a batch of
-          // HB steps has all its slices in flight before any is used (HB = sigma_max, or
-          // half of it for 32-byte slices, which would not fit the registers)
-          const uint32_t rk = c_ok ? rm : 0u;
-          VT sum = V::zero(), head = V::zero();
-          int ndk = 0;
-#pragma unroll
-          for (int k0 = 0; k0 < kSigmaMax; k0 += HB) {
-            VT xv[HB];
-            float wv[HB];
-            int nd_b = ndk;
-#pragma unroll
-            for (int u = 0; u < HB; ++u) {
-              const int k = k0 + u;
-              xv[u] = V::zero();
-              wv[u] = 0.f;
-              if ((rk >> k) & 1u) xv[u] = gather(xo + k - nd_b, wv[u]);
-              nd_b += (int)((dm >> k) & 1u);
-            }
-#pragma unroll
-            for (int u = 0; u < HB; ++u) {
-              const int k = k0 + u;
-              V::fma(wv[u], xv[u], sum);         // zero at down steps and past the lane
-              if ((dm >> k) & 1u) {
-                if (ndk == 0) head = sum;
-                else if (c_ok) epi.row(y_ws + y0 + ndk, c, sum);
-                sum = V::zero();
-                ++ndk;
-              }
-            }
-          }
-          // runs across the pass's lanes: OC_l = run open after lane l obeys
-          // OC_l = a_l + b_l * OC_{l-1} (a_l = the lane's trailing sum, b_l = 1 when the
-          // lane ends no row), with OC_{-1} = carry; scanned in log2(L) shuffle steps
-          const bool hd = dm != 0u;
-          VT A = sum;
-          int B = hd ? 0 : 1;
-          if (gl == 0) {
-            if (B) V::add(A, carry);
-            B = 0;
-          }
-#pragma unroll
-          for (int dd = 1; dd < L; dd <<= 1) {
-            const VT Ap = V::shfl_up(A, dd * T);
-            const int Bp = __shfl_up_sync(0xffffffffu, B, dd * T);
-            if (gl >= dd) {
-              if (B) V::add(A, Ap);
-              B &= Bp;
-            }
-          }
-          const VT up = V::shfl_up(A, T);
-          if (hd) {
-            VT tot = head;
-            V::add(tot, gl == 0 ? carry : up);
-            emit(y_ws + y0, tot, false);
-          }
-          const int src = (L - 1) * T + (lane % T);
-          carry = V::shfl(A, src);
-          open_row = y_ws + __shfl_sync(0xffffffffu, y0 + __popc(dm), src);
-        }
-        if (gl == L - 1) emit(open_row, carry, true);
-      };
-      if (in.endv >= in.x_be) walk(std::integral_constant<bool, true>{});
-      else walk(std::integral_constant<bool, false>{});
-    }
-    // arrival: this warp's reads of the stage and its table entries are done
-    fence_proxy_async_smem();
-    __syncwarp();
-    int last = 0;
-    if (lane == 0) {
-      __threadfence_block();
-      last = atomicAdd(&arrive[s], 1) == kWarps - 1;
-    }
-    last = __shfl_sync(0xffffffffu, last, 0);
-    if (last) {
-      __threadfence_block();
-      // rows spread over several warps of the block (never a boundary row): the table's
-      // first entry of each row adds up the row's entries
-      for (int e = gl; e < NE; e += L) {
-        const int r = wrow[e];
-        if (r < 0 || !c_ok) continue;
-        int prev = e - 1;
-        while (prev >= 0 && wrow[prev] < 0) --prev;
-        if (prev >= 0 && wrow[prev] == r) continue;      // not the first entry of its row
-        float tot[VW];
-#pragma unroll
-        for (int q = 0; q < VW; ++q) tot[q] = 0.f;
-        for (int q = e; q < NE; ++q) {
-          const int rq = wrow[q];
-          if (rq < 0) continue;
-          if (rq != r) break;
-#pragma unroll
-          for (int u = 0; u < VW; ++u) tot[u] += wval[q][c + u];
-        }
-        epi.row(r, c, V::from(tot));
+    const WalkSpan<int32_t> span(xs, xe, g.nnz);   // columns and values: both 4 bytes wide
+    if (span.end < xe) {
+      // the arrays' last nonzeros, short of a whole 16-byte unit
+      for (int k = span.end + lane; k < xe; k += 32) {
+        sc[k - span.a0] = __ldg(g.col + k);
+        sv[k - span.a0] = __ldg(vals + k);
       }
       __syncwarp();
-      if (lane == 0) {
-        arrive[s] = 0;
-        const int vn = v + S * G;
-        if (vn < g.nb) {
-          int xb, xe; uint32_t yb, ye;
-          geom_of(vn, xb, xe, yb, ye);
-          issue(s, xb, xe, yb, ye);
+    }
+    const int pad = xs - span.a0;
+    auto columns_read = [&]() {
+      // every gather's address has been formed: the column buffer takes the next tile
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (tn >= 0) issue(g.col, sc, nmeta, 0);
+    };
+
+    const bool any = xe > xs;                      // the tile has nonzeros (the same in every lane)
+    const int col0 = any ? sc[pad] : 0;
+    if (tys & kMsb) {
+      // one row: lane gl takes every L-th nonzero, the lanes' sums are added across the warp
+      const int ntile = xe - xs;
+      VT sum = V::zero();
+#pragma unroll 1
+      for (int b0 = gl; b0 - gl < ntile; b0 += L * U1) {
+        VT xv[U1];
+#pragma unroll
+        for (int u = 0; u < U1; ++u) spmm_load(x_row(b0 + u * L < ntile ? sc[pad + b0 + u * L] : col0), xv[u]);
+#pragma unroll
+        for (int u = 0; u < U1; ++u)
+          if (b0 + u * L < ntile) V::fma(sv[pad + b0 + u * L], xv[u], sum);
+      }
+      columns_read();
+#pragma unroll
+      for (int o = T; o < 32; o <<= 1) V::add(sum, V::shfl_xor(sum, o));
+      if (gl == 0) {
+        V::add(sum, V::load_shared(s_carry));
+        V::store_shared(s_carry, sum);
+      }
+    } else {
+#pragma unroll 1
+      for (int p = 0; p < T; ++p) {
+        const int l = p * L + gl;
+        const uint32_t d = __shfl_sync(0xffffffffu, desc, l);
+        const int j = t * kOmega + l;
+        const int len = j < g.lane_num ? min(g.sigma, g.steps - j * g.sigma) : 0;
+        const uint32_t valid = (1u << len) - 1u;
+        const uint32_t dm = (d >> 18) & valid;                 // down steps
+        const uint32_t rm = ~(d >> 18) & valid;                // right steps
+        const uint32_t first = dm & (0u - dm);                 // the lane's first down step
+        const int i0 = pad + (int)(d & 511u);
+        const int y0 = y_ws + (int)((d >> 9) & 511u);          // row of the first down step
+        const int32_t* cp = sc + i0;
+        const float* vp = sv + i0;
+        float* yp = y_row(y0);                                 // the row that ends next
+        VT sum = V::zero();
+        VT xv[kSigmaMax];
+        if (any) {
+#pragma unroll
+          for (int k = 0; k < kSigmaMax; ++k) {
+            const int col = cp[k];                             // step k takes nonzero k - downs before
+            spmm_load(x_row((rm >> k) & 1u ? col : col0), xv[k]);
+            if ((dm >> k) & 1u) --cp;
+          }
         }
+        if (p == T - 1) columns_read();
+        // the walk tests the masks anew: bits kept from the gathers would hold 28 registers
+        uint32_t rw = rm, dw = dm;
+        asm volatile("" : "+r"(rw), "+r"(dw));
+#pragma unroll
+        for (int k = 0; k < kSigmaMax; ++k) {
+          const float w = vp[k];
+          if ((rw >> k) & 1u) V::fma(w, xv[k], sum);
+          V::store_shared_if(first & (1u << k), s_head, sum);
+          spmm_store_if<VW, YVEC, SCALED>((dw ^ first) & c_ok & (1u << k), yp, sum, out.scale, left);
+          if ((dw >> k) & 1u) {
+            sum = V::zero();
+            yp += out.ldy;
+            --vp;
+          }
+        }
+        // inclusive scan of the open runs over the pass's lanes (threads of one slice are T
+        // apart); a lane that ends a row starts a new run
+        const bool hd = dm != 0u;
+        __syncwarp();
+        VT in = V::load_shared(s_carry);                       // the run that reaches this lane
+        if (gl == 0 && !hd) V::add(sum, in);
+        const uint32_t slice = (uint32_t)(0xffffffffull / ((1ull << T) - 1ull)) << (lane % T);   // this slice's threads
+        const uint32_t heads = __ballot_sync(0xffffffffu, hd);
+        const uint32_t upto = heads & slice & (0xffffffffu >> (31 - lane));
+        const int dist = (upto ? lane - (31 - __clz(upto)) : lane) / T;
+        uint32_t run = ~heads & (T < 32 ? ~((1u << (T & 31)) - 1u) : 0u);   // threads that continue a run
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) {
+          if (run == 0u) break;                                // no run is longer
+          const VT up = V::shfl_up(sum, o * T);
+          if (o <= dist) V::add(sum, up);
+          run &= run >> (o * T);
+        }
+        if constexpr (L > 1) {
+          const VT up = V::shfl_up(sum, T);
+          if (gl > 0) in = up;
+        }
+        if (hd) {
+          V::add(in, V::load_shared(s_head));
+          if (y0 == y_unit) {
+            if (c_ok) add_acc(t_start, in);
+          } else {
+            spmm_store_if<VW, YVEC, SCALED>(c_ok, y_row(y0), in, out.scale, left);
+          }
+        }
+        __syncwarp();
+        if (gl == L - 1) V::store_shared(s_carry, sum);
       }
     }
-    if (++s == S) {
-      s = 0;
-      par ^= 1u;
+    __syncwarp();
+    if (next_unit) {
+      const int y_end = (int)(__shfl_sync(0xffffffffu, meta, 3) & ~kMsb);
+      if (gl == 0) {
+        if (c_ok && y_end < g.n_rows) add_acc(t + 1, V::load_shared(s_carry));
+        V::store_shared(s_carry, V::zero());
+      }
+      if (tn < 0) break;
+      ++rd;
+      t_start = tn;
+      y_unit = (int)(__shfl_sync(0xffffffffu, nmeta, 2) & ~kMsb);
     }
+    // every lane has read its values: the value buffer takes the next tile
+    fence_proxy_async_smem();
+    __syncwarp();
+    issue(vals, sv, nmeta, 1);
+    t = tn;
+    meta = nmeta;
+    desc = ndesc;
+    par ^= 1u;
   }
 }
 
-// Boundary rows of the column chunk: Y[r, c] = acc[slot][c], accumulator cleared.
-template <int KC, typename Epi>
-__global__ void __launch_bounds__(256) merbit_spmm_finalize_kernel(const Geometry g,
-                                                                   const SpmmGeometry sg, Epi epi) {
-  if (epi.skip(g.red)) return;
-  const int stride = gridDim.x * blockDim.x;
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < (g.nb + 1) * KC; p += stride) {
-    const int k = p / KC, cc = p % KC;
-    if (cc >= sg.kc || __ldg(g.bnd_slot + k) != k) continue;
-    const int r = __ldg(g.bnd_row + k);
-    if (r >= g.n_rows) continue;
-    double* a = sg.acc + (size_t)k * KC + cc;
+// Rows of the unit boundaries: Y[r, c] = scale * acc[set][c], accumulator cleared.  Every
+// distinct row is written once, by its first boundary.
+template <int KC>
+__global__ void __launch_bounds__(256) merbit_spmm_finalize_kernel(const Geometry g, double* __restrict__ acc,
+                                                                   SpmmOut out) {
+  if (out.skip(g.red)) return;
+  const int c = g.unit;
+  const int nbnd = (g.tile_num + c - 1) / c + 1;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < (int64_t)nbnd * KC; p += stride) {
+    const int k = (int)(p / KC), cc = (int)(p % KC);
+    const int r = (int)(__ldg(g.tile_y + min(k * c, g.tile_num)) & ~kMsb);
+    const int prev = k > 0 ? (int)(__ldg(g.tile_y + (k - 1) * c) & ~kMsb) : -1;
+    if (cc >= out.kc || r == prev || r >= g.n_rows) continue;
+    double* a = acc + p;
     const double tot = *a;
     *a = 0.0;
-    epi.row64(r, cc, tot);
+    out.y[(int64_t)r * out.ldy + cc] = static_cast<float>(static_cast<double>(out.scale) * tot);
   }
 }
 
-template <int KC, int VW, typename Epi>
-cudaError_t launch_spmm(const merbit_plan_s* p, const float* vals, const float* X, int ldx,
-                        const SpmmGeometry& sg, const Epi& epi, cudaStream_t st) {
+// Resident CTAs (of 4 warps) per SM: 16 warps of 128 registers hold 14 slices a thread.  Batches
+// of 7 slices at 20 warps took the same time for k <= 8 and 5 % more for k = 32; 12 warps took
+// 10 % more for k = 32.  Slices of 8 columns (one 32-byte load) need 168 registers: k = 32 took
+// 0.538 ms against 0.466 ms (R-MAT scale 21).
+template <int VW>
+constexpr int kSpmmCtas = VW == 4 ? 4 : 7;
+
+// Unit length and the number of accumulator sets (unit boundaries) of a plan's SpMM.
+inline int spmm_unit(const merbit_plan_s* p) { return walk_unit(p->tile_num, (int64_t)p->num_sms * 16, kTilesPerBlock); }
+inline int64_t spmm_sets(const merbit_plan_s* p) {
+  const int c = spmm_unit(p);
+  return (p->tile_num + c - 1) / c + 1;
+}
+
+template <int KC, int VW, bool YVEC, bool SCALED>
+cudaError_t launch_spmm(const merbit_plan_s* p, const float* vals, const float* X, int64_t ldx, const SpmmOut& out,
+                        double* acc, cudaStream_t st) {
   if (p->nb == 0) return cudaSuccess;
-  auto kern = merbit_spmm_kernel<KC, VW, Epi>;
+  auto kern = merbit_spmm_kernel<KC, VW, YVEC, SCALED, kSpmmCtas<VW>>;
   const void* kp = reinterpret_cast<const void*>(kern);
-  const size_t smem = kSpmmStages * stage_bytes<float>(p->sigma, kTilesPerBlock);
-  const size_t smem_max = kSpmmStages * stage_bytes<float>(kSigmaMax, kTilesPerBlock);
-  int grid = persistent_grid(kp, kThreads, smem, smem_max, p->num_sms);
+  const size_t smem = kSpmmWarps * spmm_warp_bytes<VW>(p->sigma);
+  int grid = persistent_grid(kp, kSpmmThreads, smem, kSpmmWarps * spmm_warp_bytes<VW>(kSigmaMax), p->num_sms);
   if (grid <= 0) return cudaErrorInvalidConfiguration;
-  if ((int64_t)grid > p->nb) grid = (int)p->nb;
-  kern<<<grid, kThreads, smem, st>>>(p->geom(), sg, vals, X, ldx, epi);
+  Geometry g = p->geom();
+  g.unit = spmm_unit(p);
+  const int64_t units = (p->tile_num + g.unit - 1) / g.unit;
+  const int64_t few = std::max<int64_t>((units + kSpmmWarps - 1) / kSpmmWarps, std::min<int64_t>(units, p->num_sms));
+  if (grid > few) grid = (int)few;
+  const int round = grid * kSpmmWarps;
+  const SpmmUnits un{(int)(units / round), (int)(units % round)};
+  kern<<<grid, kSpmmThreads, smem, st>>>(g, un, acc, vals, X, ldx, out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int64_t work = (p->nb + 1) * KC;
+  const int64_t work = (units + 1) * KC;
   const int fgrid = (int)std::min<int64_t>((work + 255) / 256, (int64_t)p->num_sms * 8);
-  merbit_spmm_finalize_kernel<KC, Epi><<<fgrid, 256, 0, st>>>(p->geom(), sg, epi);
+  merbit_spmm_finalize_kernel<KC><<<fgrid, 256, 0, st>>>(g, acc, out);
   return cudaGetLastError();
 }
 
