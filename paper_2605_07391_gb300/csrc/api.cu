@@ -60,14 +60,7 @@ void free_plan(merbit_plan_s* p) {
   if (!p) return;
   host_async_release(p);
   free_hot_table(p);
-  cudaFree(p->tile_x);
-  cudaFree(p->tile_y);
-  cudaFree(p->lane_desc);
-  cudaFree(p->bnd_row);
-  cudaFree(p->bnd_slot);
-  cudaFree(p->bnd_acc);
-  cudaFree(p->part);
-  cudaFree(p->red);
+  cudaFree(p->block);
   cudaFree(p->dangling_bits);
   cudaFree(p->scratch);
   cudaFree(p->hist);
@@ -79,21 +72,23 @@ void free_plan(merbit_plan_s* p) {
   delete p;
 }
 
-cudaError_t grow(void** buf, size_t* cap, size_t need) {
+cudaError_t grow(void** buf, size_t* cap, size_t need, cudaStream_t st) {
   if (*cap >= need) return cudaSuccess;
-  cudaFree(*buf);
+  if (*buf) {
+    cudaDeviceSynchronize();   // earlier calls may still use it
+    cudaFree(*buf);
+  }
   *buf = nullptr;
   *cap = 0;
-  cudaError_t e = cudaMalloc(buf, need);
+  cudaError_t e = dev_alloc(buf, need, st);
   if (e == cudaSuccess) *cap = need;
   return e;
 }
 
 cudaError_t reset_device_state(merbit_plan_s* p, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(p->red, 0, sizeof(RedState), st);
-  // the tile accumulators follow the block accumulators
-  if (e == cudaSuccess && p->nb > 0)
-    e = cudaMemsetAsync(p->bnd_acc, 0, sizeof(double) * (size_t)(p->nb + 1 + p->tile_num + 1), st);
+  // the state and the block and tile accumulators lie one behind the other
+  char* const end = reinterpret_cast<char*>(p->tile_acc + (p->tile_num + 1));
+  cudaError_t e = cudaMemsetAsync(p->red, 0, (size_t)(end - reinterpret_cast<char*>(p->red)), st);
   if (e == cudaSuccess && p->spmm_acc)
     e = cudaMemsetAsync(p->spmm_acc, 0, sizeof(double) * 32 * (size_t)spmm_acc_sets(p), st);
   return e;
@@ -103,6 +98,10 @@ cudaError_t reset_device_state(merbit_plan_s* p, cudaStream_t st) {
 struct StateWord { int err, done, iters, inner_done, launches; };
 
 cudaError_t read_state(merbit_plan_s* p, cudaStream_t st, StateWord* w) {
+  if (!p->host_pinned) {
+    const cudaError_t h = cudaMallocHost(&p->host_pinned, 256);
+    if (h != cudaSuccess) return h;
+  }
   cudaError_t e = cudaMemcpyAsync(p->host_pinned, &p->red->err, sizeof(StateWord),
                                   cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -260,14 +259,14 @@ merbit_status ensure_dangling(merbit_plan_s* p, cudaStream_t st) {
   return MERBIT_OK;
 }
 
-merbit_status ensure_hist(merbit_plan_s* p, size_t launches) {
+merbit_status ensure_hist(merbit_plan_s* p, size_t launches, cudaStream_t st) {
   const size_t need = 2 * (launches + 2);
-  if (p->hist_len >= need) return MERBIT_OK;
-  cudaFree(p->hist);
-  p->hist = nullptr;
-  p->hist_len = 0;
-  MB_TRY(cudaMalloc(&p->hist, need * sizeof(double)));
-  p->hist_len = need;
+  size_t cap = p->hist_len * sizeof(double);
+  void* buf = p->hist;
+  const cudaError_t e = grow(&buf, &cap, need * sizeof(double), st);
+  p->hist = static_cast<double*>(buf);
+  p->hist_len = cap / sizeof(double);
+  MB_TRY(e);
   return MERBIT_OK;
 }
 
@@ -335,7 +334,11 @@ merbit_status merbit_plan_ex(const int32_t* row_ptr, const int32_t* col_idx, int
   }
 
   merbit_plan_s* p = new merbit_plan_s();
-  auto bail = [&](merbit_status s) { free_plan(p); return s; };
+  auto bail = [&](merbit_status s) {
+    cudaDeviceSynchronize();
+    free_plan(p);
+    return s;
+  };
   cudaGetDevice(&p->device);
   cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device);
   p->n_rows = n_rows;
@@ -350,26 +353,34 @@ merbit_status merbit_plan_ex(const int32_t* row_ptr, const int32_t* col_idx, int
   p->tile_num = (steps + (int64_t)kOmega * sigma - 1) / ((int64_t)kOmega * sigma);
   p->nb = (p->tile_num + tiles_per_block - 1) / tiles_per_block;
 
-  cudaError_t e = cudaSuccess;
+  // one block for the plan's arrays; the state and the accumulators come last, to be cleared at once
+  size_t bytes = 0;
+  const auto place = [&](size_t b) {
+    const size_t at = bytes;
+    bytes += (b + 255) & ~size_t(255);
+    return at;
+  };
   const size_t tb = sizeof(uint32_t) * (size_t)(p->tile_num + 1);
   const size_t nbb = sizeof(int32_t) * (size_t)(p->nb + 1);
-  if (e == cudaSuccess) e = cudaMalloc(&p->tile_x, tb);
-  if (e == cudaSuccess) e = cudaMalloc(&p->tile_y, tb);
-  if (e == cudaSuccess)
-    e = cudaMalloc(&p->lane_desc, (size_t)p->desc_bytes * (size_t)std::max<int64_t>(p->lane_num, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_row, nbb);
-  // the tile slots and accumulators lie behind the block ones, in the same allocations
-  const size_t bounds = (size_t)(p->nb + 1) + (size_t)(p->tile_num + 1);
-  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_slot, sizeof(int32_t) * bounds);
-  if (e == cudaSuccess) e = cudaMalloc(&p->bnd_acc, sizeof(double) * bounds);
-  if (e == cudaSuccess) {
-    p->tile_slot = p->bnd_slot + (p->nb + 1);
-    p->tile_acc = p->bnd_acc + (p->nb + 1);
-  }
-  if (e == cudaSuccess) e = cudaMalloc(&p->part, sizeof(double2) * (size_t)kMaxParts);
-  if (e == cudaSuccess) e = cudaMalloc(&p->red, sizeof(RedState));
-  if (e == cudaSuccess) e = cudaMallocHost(&p->host_pinned, 256);
+  const size_t at_x = place(tb), at_y = place(tb);
+  const size_t at_desc = place((size_t)p->desc_bytes * (size_t)std::max<int64_t>(p->lane_num, 1));
+  const size_t at_row = place(nbb), at_bslot = place(nbb), at_tslot = place(tb);
+  const size_t at_part = place(sizeof(double2) * (size_t)kMaxParts);
+  const size_t at_red = place(sizeof(RedState));
+  const size_t at_acc = place(sizeof(double) * (size_t)((p->nb + 1) + (p->tile_num + 1)));
+  cudaError_t e = dev_alloc(&p->block, bytes, st);
   if (e != cudaSuccess) return bail(cuda_fail(e, "plan allocation"));
+  char* const mem = static_cast<char*>(p->block);
+  p->tile_x = reinterpret_cast<uint32_t*>(mem + at_x);
+  p->tile_y = reinterpret_cast<uint32_t*>(mem + at_y);
+  p->lane_desc = reinterpret_cast<uint32_t*>(mem + at_desc);
+  p->bnd_row = reinterpret_cast<int32_t*>(mem + at_row);
+  p->bnd_slot = reinterpret_cast<int32_t*>(mem + at_bslot);
+  p->tile_slot = reinterpret_cast<int32_t*>(mem + at_tslot);
+  p->part = reinterpret_cast<double2*>(mem + at_part);
+  p->red = reinterpret_cast<RedState*>(mem + at_red);
+  p->bnd_acc = reinterpret_cast<double*>(mem + at_acc);
+  p->tile_acc = p->bnd_acc + (p->nb + 1);
   if (p->tile_num == 0) {
     // empty path (n_rows = 0): only the terminator
     const uint32_t term[2] = {(uint32_t)nnz, (uint32_t)n_rows};
@@ -547,13 +558,13 @@ merbit_status merbit_ppr(merbit_plan_t p, const float* vals, const int32_t* seed
     if (seeds[c] < 0 || seeds[c] >= n) return fail(MERBIT_EINVAL, "seed %lld out of range", (long long)c);
   cudaStream_t st = as_stream(stream);
   if (merbit_status s = ensure_dangling(p, st)) return s;
-  if (merbit_status s = ensure_hist(p, (size_t)max_iter)) return s;
+  if (merbit_status s = ensure_hist(p, (size_t)max_iter, st)) return s;
   if (merbit_status s = ensure_spmm_acc(p, st)) return s;
   // scratch: second iterate | seeds | D per column | 2k accumulators | last residuals
   const size_t xb = align256(sizeof(float) * (size_t)n * (size_t)k);
   const size_t sb = align256(sizeof(int32_t) * (size_t)k);
   const size_t db = align256(sizeof(double) * (size_t)k);
-  MB_TRY(grow(&p->scratch, &p->scratch_bytes, xb + sb + 4 * db));
+  MB_TRY(grow(&p->scratch, &p->scratch_bytes, xb + sb + 4 * db, st));
   char* base = static_cast<char*>(p->scratch);
   float* x1 = reinterpret_cast<float*>(base);
   int32_t* seed_d = reinterpret_cast<int32_t*>(base + xb);
@@ -610,8 +621,8 @@ merbit_status merbit_spmv_host(merbit_plan_t p, merbit_dtype dtype, const void* 
   cudaStream_t st = as_stream(stream);
   const size_t es = dtype_size(dtype);
   const size_t xb = es * (size_t)p->n_cols, yb = es * (size_t)p->n_rows;
-  MB_TRY(grow(&p->x_stage, &p->x_stage_bytes, std::max<size_t>(xb, 16)));
-  MB_TRY(grow(&p->y_stage, &p->y_stage_bytes, std::max<size_t>(yb, 16)));
+  MB_TRY(grow(&p->x_stage, &p->x_stage_bytes, std::max<size_t>(xb, 16), st));
+  MB_TRY(grow(&p->y_stage, &p->y_stage_bytes, std::max<size_t>(yb, 16), st));
   if (xb) MB_TRY(cudaMemcpyAsync(p->x_stage, x_host, xb, cudaMemcpyHostToDevice, st));
   merbit_status s = merbit_spmv_ex(p, dtype, dtype, vals, p->x_stage, p->y_stage, 0, stream);
   if (s != MERBIT_OK) return s;
@@ -645,8 +656,8 @@ merbit_status pagerank_plain(merbit_plan_s* p, const T* vals, double alpha, doub
                              int max_iter, T* pi, int* iters_out, double* resid_out,
                              double* resid_hist, int* launches_out, cudaStream_t st) {
   const int64_t n = p->n_rows;
-  MB_TRY(grow(&p->scratch, &p->scratch_bytes, align256(sizeof(T) * (size_t)n)));
-  if (merbit_status s = ensure_hist(p, (size_t)max_iter)) return s;
+  MB_TRY(grow(&p->scratch, &p->scratch_bytes, align256(sizeof(T) * (size_t)n), st));
+  if (merbit_status s = ensure_hist(p, (size_t)max_iter, st)) return s;
   T* buf[2] = {pi, static_cast<T*>(p->scratch)};
   const double d0 = (double)p->n_dangling / (double)n;
   fill_kernel<T><<<grid_for(n, p->num_sms), 256, 0, st>>>(pi, n, static_cast<T>(1.0 / (double)n));
@@ -714,7 +725,7 @@ merbit_status pagerank_ir(merbit_plan_s* p, const double* vals, double alpha, do
                      : ldt == MERBIT_F16 ? std::ldexp(1.0, -11) : std::ldexp(1.0, -17);
   const size_t lo_bytes = align256(dtype_size(ldt) * (size_t)std::max<int64_t>(p->nnz, 1));
   const size_t vb = align256(sizeof(float) * (size_t)n);
-  MB_TRY(grow(&p->scratch, &p->scratch_bytes, lo_bytes + 3 * vb));
+  MB_TRY(grow(&p->scratch, &p->scratch_bytes, lo_bytes + 3 * vb, st));
   char* base = static_cast<char*>(p->scratch);
   void* lo = base;
   float* rhs = reinterpret_cast<float*>(base + lo_bytes);
@@ -725,7 +736,7 @@ merbit_status pagerank_ir(merbit_plan_s* p, const double* vals, double alpha, do
                                       p->num_sms))
     return s;
   const size_t per_step = (size_t)max_sweeps + 2;
-  if (merbit_status s = ensure_hist(p, ((size_t)max_steps + 1) * per_step + 1)) return s;
+  if (merbit_status s = ensure_hist(p, ((size_t)max_steps + 1) * per_step + 1, st)) return s;
   const double d0 = (double)p->n_dangling / (double)n;
   fill_kernel<double><<<grid_for(n, p->num_sms), 256, 0, st>>>(pi, n, 1.0 / (double)n);
   pr_state_init_kernel<<<1, 1, 0, st>>>(p->hist, d0, p->red);
@@ -880,9 +891,9 @@ merbit_status merbit_pagerank_adjoint(merbit_plan_t p, merbit_plan_t pt, merbit_
     return fail(MERBIT_EINVAL, "vals_t must be a 16-byte aligned device array");
   cudaStream_t st = as_stream(stream);
   if (merbit_status s = ensure_dangling(p, st)) return s;
-  if (merbit_status s = ensure_hist(pt, (size_t)max_iter)) return s;
+  if (merbit_status s = ensure_hist(pt, (size_t)max_iter, st)) return s;
   const size_t es = dtype_size(dtype);
-  MB_TRY(grow(&pt->scratch, &pt->scratch_bytes, align256(es * (size_t)n) + 256));
+  MB_TRY(grow(&pt->scratch, &pt->scratch_bytes, align256(es * (size_t)n) + 256, st));
   void* buf[2] = {lambda, pt->scratch};
   double* wnorm = reinterpret_cast<double*>(static_cast<char*>(pt->scratch) + align256(es * (size_t)n));
   // lambda_0 = w, S_0 = sum(w); state cleared

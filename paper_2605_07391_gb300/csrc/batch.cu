@@ -557,7 +557,7 @@ merbit_status merbit_batch_plan(const int32_t* row_ptr, const int32_t* col_idx, 
   for (int g = 0; g < num_graphs; ++g) inv_n[g] = 1.0 / (double)(graph_offsets[g + 1] - graph_offsets[g]);
   const size_t G = (size_t)num_graphs;
   cudaError_t e = cudaSuccess;
-  auto A = [&](void** q, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(q, bytes); };
+  auto A = [&](void** q, size_t bytes) { if (e == cudaSuccess) e = dev_alloc(q, bytes, st); };
   A((void**)&b->off, sizeof(int32_t) * (G + 1));
   A((void**)&b->inv_n, sizeof(double) * G);
   A((void**)&b->dang0, sizeof(double) * G);
@@ -599,6 +599,7 @@ merbit_status merbit_batch_plan(const int32_t* row_ptr, const int32_t* col_idx, 
   std::vector<double> d0(G);
   for (size_t g = 0; g < G; ++g) d0[g] = (double)cnt_h[g] * inv_n[g];
   if (e == cudaSuccess) e = cudaMemcpy(b->dang0, d0.data(), sizeof(double) * G, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) cudaDeviceSynchronize();   // nothing may use the blocks that go
   cudaFree(cnt);
   cudaFree(err);
   if (e != cudaSuccess) {

@@ -220,8 +220,9 @@ merbit_status merbit_bicgstab(merbit_plan_t p, const double* vals, const double*
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t vb = (sizeof(double) * (size_t)n + 255) & ~size_t(255);
   const size_t sb = (sizeof(BicgState) + 255) & ~size_t(255);
-  char* mem = nullptr;
-  cudaError_t e = cudaMalloc(&mem, 6 * vb + sb + sizeof(double) * (size_t)max_iter);
+  void* block = nullptr;
+  cudaError_t e = dev_alloc(&block, 6 * vb + sb + sizeof(double) * (size_t)max_iter, st);
+  char* const mem = static_cast<char*>(block);
   if (e != cudaSuccess) return bfail2(e == cudaErrorMemoryAllocation ? MERBIT_ENOMEM : MERBIT_ECUDA,
                                       "BiCGSTAB work vectors");
   BicgVecs w;
@@ -303,6 +304,7 @@ merbit_status merbit_bicgstab(merbit_plan_t p, const double* vals, const double*
   if (exec) cudaGraphExecDestroy(exec);
   if (graph) cudaGraphDestroy(graph);
   if (cap) cudaStreamDestroy(cap);
+  if (e != cudaSuccess) cudaDeviceSynchronize();   // nothing may use the block that goes
   cudaFree(mem);
   if (e != cudaSuccess) {
     char msg[256];

@@ -77,6 +77,7 @@ struct merbit_plan_s {
   uint32_t wait_limit = merbit::kSpinLimit;   // polls of a stage wait (test hook lowers it)
   int64_t tile_num = 0, lane_num = 0, nb = 0;
   const int32_t* col = nullptr;          // borrowed
+  void* block = nullptr;                 // the plan's own arrays below, up to red, in one allocation
   // hot-column table: col_hot is a copy of col in which a column held in the table is
   // replaced by ~slot; hot_list[slot] is that column (slots by decreasing use)
   int32_t* col_hot = nullptr;
@@ -88,8 +89,8 @@ struct merbit_plan_s {
   uint32_t* lane_desc = nullptr;
   int32_t* bnd_row = nullptr;
   int32_t* bnd_slot = nullptr;
-  double* bnd_acc = nullptr;
-  int32_t* tile_slot = nullptr;          // tile_num + 1, behind bnd_slot; null: no lane-walk kernel
+  double* bnd_acc = nullptr;             // directly behind red; tile_acc directly behind it
+  int32_t* tile_slot = nullptr;          // tile_num + 1; null: no lane-walk kernel
   double* tile_acc = nullptr;            // tile_num + 1, behind bnd_acc
   double2* part = nullptr;               // kMaxParts entries
   merbit::RedState* red = nullptr;
@@ -104,7 +105,7 @@ struct merbit_plan_s {
   void* x_stage = nullptr;               // staging for host-buffer SpMV
   void* y_stage = nullptr;
   size_t x_stage_bytes = 0, y_stage_bytes = 0;
-  void* host_pinned = nullptr;           // small pinned block for state read-back
+  void* host_pinned = nullptr;           // small pinned block for state read-back (on first use)
   double* spmm_acc = nullptr;            // spmm_acc_sets x 32 FP64 boundary accumulators of the SpMM
   void* spmm_pack = nullptr;             // padded copy of up to 32 columns of an unaligned X
   size_t spmm_pack_bytes = 0;
@@ -177,6 +178,10 @@ struct SweepParams {
   const double* rnorm;          // ||r||_1 of the current refinement step
   double eta;                   // inner stop: sweep size <= eta * ||r||_1
 };
+
+// A block of device memory from the library's pool (memory.cu); freed by cudaFree after the work
+// that uses it has been waited for.
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
 
 // ---- launchers (one translation unit per value type) ----
 cudaError_t spmv_plain_f32(const merbit_plan_s* p, const float* vals, const float* x, float* y,

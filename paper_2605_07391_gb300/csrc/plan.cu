@@ -150,16 +150,19 @@ cudaError_t build_tiles(const merbit_plan_s* p, const int32_t* row_ptr, cudaStre
 
 cudaError_t build_dangling(merbit_plan_s* p, cudaStream_t st, unsigned long long* host_count) {
   const int n = (int)p->n_cols;
-  uint8_t* present = nullptr;
-  unsigned long long* cnt = nullptr;
-  cudaError_t e = cudaMalloc(&present, (size_t)n + 8);
+  // the columns' marks and the count in one block
+  const size_t at = ((size_t)n + 255) & ~size_t(255);
+  void* mem = nullptr;
+  cudaError_t e = dev_alloc(&mem, at + sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  e = cudaMalloc(&cnt, sizeof(unsigned long long));
-  if (e != cudaSuccess) { cudaFree(present); return e; }
+  uint8_t* const present = static_cast<uint8_t*>(mem);
+  unsigned long long* const cnt = reinterpret_cast<unsigned long long*>(present + at);
   const size_t words = ((size_t)n + 31) / 32;
   if (!p->dangling_bits) {
-    e = cudaMalloc(&p->dangling_bits, words * sizeof(uint32_t) + 4);
-    if (e != cudaSuccess) { cudaFree(present); cudaFree(cnt); return e; }
+    void* bits = nullptr;
+    e = dev_alloc(&bits, words * sizeof(uint32_t) + 4, st);
+    if (e != cudaSuccess) { cudaFree(mem); return e; }
+    p->dangling_bits = static_cast<uint32_t*>(bits);
   }
   cudaMemsetAsync(present, 0, (size_t)n, st);
   cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st);
@@ -171,10 +174,9 @@ cudaError_t build_dangling(merbit_plan_s* p, cudaStream_t st, unsigned long long
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(host_count, cnt, sizeof(unsigned long long),
                                             cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(present);
-  cudaFree(cnt);
-  return e;
+  const cudaError_t es = cudaStreamSynchronize(st);
+  cudaFree(mem);
+  return e == cudaSuccess ? es : e;
 }
 
 int persistent_grid(const void* kernel, int threads, size_t smem, size_t smem_max, int num_sms) {

@@ -384,10 +384,10 @@ cudaError_t build_transpose(merbit_transpose_s* t, const int32_t* row_ptr, const
   const size_t hb = up(sizeof(uint32_t) * (size_t)bins * (size_t)num_tiles);
   const size_t tb = up(sizeof(uint32_t) * (size_t)bins);
   const int sets = passes > 2 ? 2 : passes - 1;
-  char* mem = nullptr;
-  cudaError_t e = cudaMalloc(&mem, (size_t)sets * (nb + pb) + nb + hb + tb + up(sizeof(int32_t) * (size_t)num_tiles));
+  void* mem = nullptr;
+  cudaError_t e = dev_alloc(&mem, (size_t)sets * (nb + pb) + nb + hb + tb + up(sizeof(int32_t) * (size_t)num_tiles), st);
   if (e != cudaSuccess) return e;
-  char* m = mem;
+  char* m = static_cast<char*>(mem);
   const auto take = [&](size_t b) {
     char* r = m;
     m += b;
@@ -434,9 +434,8 @@ cudaError_t build_transpose(merbit_transpose_s* t, const int32_t* row_ptr, const
 
 void free_transpose(merbit_transpose_s* t) {
   if (!t) return;
-  cudaFree(t->row_ptr_t);
-  cudaFree(t->col_t);
-  cudaFree(t->perm);
+  cudaDeviceSynchronize();   // work that reads the arrays
+  cudaFree(t->row_ptr_t);    // the three arrays' block
   delete t;
 }
 
@@ -479,9 +478,15 @@ merbit_status merbit_transpose(const int32_t* row_ptr, const int32_t* col_idx, i
   t->n_cols = n_cols;
   t->nnz = nnz;
   cudaGetDevice(&t->device);
-  cudaError_t e = cudaMalloc(&t->row_ptr_t, sizeof(int32_t) * (size_t)(n_cols + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&t->col_t, sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&t->perm, sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1));
+  const size_t pb = (sizeof(int32_t) * (size_t)(n_cols + 1) + 255) & ~size_t(255);
+  const size_t nb = (sizeof(int32_t) * (size_t)std::max<int64_t>(nnz, 1) + 255) & ~size_t(255);
+  void* mem = nullptr;
+  cudaError_t e = dev_alloc(&mem, pb + 2 * nb, static_cast<cudaStream_t>(stream));
+  if (e == cudaSuccess) {
+    t->row_ptr_t = static_cast<int32_t*>(mem);
+    t->col_t = reinterpret_cast<int32_t*>(static_cast<char*>(mem) + pb);
+    t->perm = reinterpret_cast<int32_t*>(static_cast<char*>(mem) + pb + nb);
+  }
   if (e == cudaSuccess) e = build_transpose(t, row_ptr, col_idx, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) {
     free_transpose(t);

@@ -66,6 +66,8 @@ def library_path() -> str:
 def load(path: str | None = None) -> ctypes.CDLL:
     """Load libmerbit.so (building it first if it is missing or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -138,18 +140,26 @@ def _check(where: str, status: int, allow: tuple[int, ...] = ()) -> int:
     return status
 
 
-def _ptr(t: torch.Tensor | None) -> ctypes.c_void_p:
+# Pointers and streams are passed as integers (the argument types convert them): a ctypes object
+# each would cost more than the conversion.
+def _ptr(t: torch.Tensor | None) -> int:
     if t is None:
-        return ctypes.c_void_p(0)
+        return 0
     if not t.is_contiguous():
         raise ValueError("tensors passed to the MERBIT library must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# the current stream's handle without a Stream object around it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _dt(t: torch.Tensor) -> int:
@@ -273,9 +283,28 @@ class _DeviceArray:
         self._owner = owner
 
 
+class _TransposeHandle:
+    """The library's transpose object.  The arrays' views hold this and not the Transpose, which
+    holds the views: a cycle through a tensor's storage is never collected."""
+
+    def __init__(self):
+        self.value = ctypes.c_void_p()
+
+    def destroy(self):
+        if self.value:
+            load().merbit_transpose_destroy(self.value)
+            self.value = ctypes.c_void_p()
+
+    def __del__(self):
+        try:
+            self.destroy()
+        except Exception:
+            pass
+
+
 class Transpose:
     """merbit_transpose: the CSR of A^T on the device (row_ptr_t, col_t, perm), owned by
-    the library; the tensors below are views that keep this object alive."""
+    the library; the tensors below are views that keep the arrays alive."""
 
     def __init__(self, row_ptr: torch.Tensor, col_idx: torch.Tensor, n_rows: int | None = None,
                  n_cols: int | None = None, stream=None):
@@ -285,18 +314,18 @@ class Transpose:
             raise ValueError("row_ptr and col_idx must be int32")
         n_rows = row_ptr.numel() - 1 if n_rows is None else n_rows
         n_cols = n_rows if n_cols is None else n_cols
-        self._handle = ctypes.c_void_p()
+        self._owner = _TransposeHandle()
         _check("merbit_transpose", lib.merbit_transpose(_ptr(row_ptr), _ptr(col_idx), n_rows, n_cols,
                                                        col_idx.numel(), _stream(stream),
-                                                       ctypes.byref(self._handle)))
+                                                       ctypes.byref(self._owner.value)))
         rp, ct, pm = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
-        _check("merbit_transpose_get", lib.merbit_transpose_get(self._handle, ctypes.byref(rp),
+        _check("merbit_transpose_get", lib.merbit_transpose_get(self._owner.value, ctypes.byref(rp),
                                                                ctypes.byref(ct), ctypes.byref(pm)))
         nnz = col_idx.numel()
         dev = row_ptr.device
-        self.row_ptr_t = torch.as_tensor(_DeviceArray(rp.value, n_cols + 1, "<i4", self), device=dev)
-        self.col_t = torch.as_tensor(_DeviceArray(ct.value, nnz, "<i4", self), device=dev)
-        self.perm = torch.as_tensor(_DeviceArray(pm.value, nnz, "<i4", self), device=dev)
+        self.row_ptr_t = torch.as_tensor(_DeviceArray(rp.value, n_cols + 1, "<i4", self._owner), device=dev)
+        self.col_t = torch.as_tensor(_DeviceArray(ct.value, nnz, "<i4", self._owner), device=dev)
+        self.perm = torch.as_tensor(_DeviceArray(pm.value, nnz, "<i4", self._owner), device=dev)
         self.n_rows, self.n_cols, self.nnz = n_cols, n_rows, nnz    # of A^T
 
     def plan(self, sigma: int = 14, stream=None) -> "Plan":
@@ -304,15 +333,7 @@ class Transpose:
         return Plan(self.row_ptr_t, self.col_t, self.n_rows, self.n_cols, sigma=sigma, stream=stream)
 
     def destroy(self):
-        if getattr(self, "_handle", None):
-            load().merbit_transpose_destroy(self._handle)
-            self._handle = ctypes.c_void_p()
-
-    def __del__(self):
-        try:
-            self.destroy()
-        except Exception:
-            pass
+        self._owner.destroy()
 
 
 class Batch:
@@ -519,8 +540,9 @@ def spmv(p: Plan, vals: torch.Tensor, x: torch.Tensor, y: torch.Tensor | None = 
     xdt = _dt(x)
     if y is None:
         y = torch.empty(p.n_rows, dtype=x.dtype, device=x.device)
-    _check("merbit_spmv_ex", load().merbit_spmv_ex(p.handle, _dt(vals), xdt, _ptr(vals), _ptr(x),
-                                                  _ptr(y), scale_exp, _stream(stream)))
+    st = load().merbit_spmv_ex(p.handle, _dt(vals), xdt, _ptr(vals), _ptr(x), _ptr(y), scale_exp, _stream(stream))
+    if st:
+        _check("merbit_spmv_ex", st)
     return y
 
 

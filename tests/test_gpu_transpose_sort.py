@@ -42,3 +42,21 @@ def test_rows_across_tiles(cuda_device):
     lens[[0, 3, 40_000, 59_999]] = [30_000, 1, 7_000, 3]
     lens[30_000:30_020] = 613
     _check(lens, rng.integers(0, 5000, lens.sum()), 5000)
+
+
+def test_dropped_transposes_give_their_memory_back(cuda_device):
+    """A transpose whose object and views are gone frees its arrays (they stay while a view lives)."""
+    n, nnz = 1000, 4_000_000
+    row_ptr = torch.arange(n + 1, dtype=torch.int32, device="cuda") * (nnz // n)
+    col = torch.randint(0, n, (nnz,), dtype=torch.int32, device="cuda")
+    first = mb.transpose(row_ptr, col).perm               # a view alone keeps the arrays
+    want = first.cpu()
+    for _ in range(3):
+        mb.transpose(row_ptr, col)
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(50):                                   # 32 MB each
+        t = mb.transpose(row_ptr, col)
+        view = t.col_t
+        del t, view
+    assert free - torch.cuda.mem_get_info()[0] < 200 << 20
+    assert torch.equal(first.cpu(), want)
