@@ -131,6 +131,7 @@ __global__ void pr_state_init_kernel(double* hist, double d0, RedState* red) {
   red->iters = 0;
   red->inner_done = 0;
   red->launches = 0;
+  red->bar = 0u;
   red->delta = nullptr;   // published again by this solve's first residual pass
 }
 
@@ -656,7 +657,9 @@ merbit_status pagerank_plain(merbit_plan_s* p, const T* vals, double alpha, doub
                              int max_iter, T* pi, int* iters_out, double* resid_out,
                              double* resid_hist, int* launches_out, cudaStream_t st) {
   const int64_t n = p->n_rows;
-  MB_TRY(grow(&p->scratch, &p->scratch_bytes, align256(sizeof(T) * (size_t)n), st));
+  const size_t xb = align256(sizeof(T) * (size_t)n);
+  MB_TRY(grow(&p->scratch, &p->scratch_bytes, xb + 2 * sizeof(double) * (size_t)p->tile_num, st));
+  double* const shares = reinterpret_cast<double*>(static_cast<char*>(p->scratch) + xb);
   if (merbit_status s = ensure_hist(p, (size_t)max_iter, st)) return s;
   T* buf[2] = {pi, static_cast<T*>(p->scratch)};
   const double d0 = (double)p->n_dangling / (double)n;
@@ -666,6 +669,13 @@ merbit_status pagerank_plain(merbit_plan_s* p, const T* vals, double alpha, doub
   const int kBatch = 8;
   int k = 0;
   StateWord w{};
+  bool resident = false;
+  MB_TRY(pagerank_resident(p, sizeof(T) == 4 ? MERBIT_F32 : MERBIT_F64, vals, alpha, tol, max_iter, buf[0], buf[1], p->hist,
+                           shares, &resident, st));
+  if (resident) {
+    MB_TRY(read_state(p, st, &w));
+    k = max_iter;
+  }
   while (k < max_iter) {
     const int stop = std::min(max_iter, k + kBatch);
     for (; k < stop; ++k) {

@@ -32,6 +32,7 @@ struct RedState {
   int iters;      // number of launches counted when `done` was set
   int inner_done; // refinement: the inner sweeps of the current step have converged
   int launches;   // SpMV launches that did work since the solve started
+  unsigned int bar;   // arrivals at the grid barriers of a cooperative solve
   const float* delta;   // refinement: buffer holding the latest inner iterate
 };
 
@@ -217,6 +218,13 @@ cudaError_t ppr_update(merbit_plan_s* p, const float* vals, const float* X, floa
                        int64_t k, const int32_t* seed, double* d_cur, double* rd, double* last_r,
                        float alpha, double tol, int iter, double* hist, double* acc,
                        cudaStream_t st);
+// All updates of a plain PageRank in one cooperative launch, from x0 (iterate k is in x0 for even k,
+// else in x1); *taken = false and nothing launched if the matrix does not fit the SMs' shared
+// memory.  hist[1] holds the first iterate's dangling mass, red->bar is zero; shares: 2 tile_num
+// doubles of work space.
+cudaError_t pagerank_resident(merbit_plan_s* p, merbit_dtype dt, const void* vals, double alpha, double tol,
+                              int max_iter, void* x0, void* x1, double* hist, double* shares, bool* taken,
+                              cudaStream_t st);
 // pi += delta (FP64) with delta = the refinement's latest inner iterate; s_out[1] = dangling mass
 cudaError_t ir_apply(const merbit_plan_s* p, double* pi, double* s_out, cudaStream_t st);
 

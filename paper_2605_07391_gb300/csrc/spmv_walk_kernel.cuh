@@ -90,6 +90,67 @@ __device__ __forceinline__ void walk_issue(const T* src, void* dst, int xs, int 
   if (bytes) bulk_g2s(dst, src + sp.a0, bytes, bar, pol);
 }
 
+// The walk of one tile by a warp: a lane's steps (rm: right steps, dm: down steps; vp its first
+// value; xv its gathered x), the row sums into sy (y0: the row of the lane's first down step), the
+// runs joined across the lanes.  carry is the run that reaches the tile; the run open after it is
+// returned, in every lane.
+template <typename VT, typename XT, typename AT>
+__device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax], uint32_t rm, uint32_t dm, AT* sy,
+                                         int y0, AT carry, int lane) {
+  const uint32_t first = dm & (0u - dm);             // the lane's first down step
+  const uint32_t later = dm ^ first;
+  AT* rp = sy + y0;
+  AT sum = AT(0), head = AT(0);
+#pragma unroll
+  for (int k = 0; k < kSigmaMax; ++k) {
+    if constexpr (!IsUnit<VT>::value) {
+      const AT v = static_cast<AT>(widen(vp[k]));
+      if ((rm >> k) & 1u) sum = mul_add(v, static_cast<AT>(xv[k]), sum);
+    } else {
+      if ((rm >> k) & 1u) sum += static_cast<AT>(xv[k]);
+    }
+    if ((first >> k) & 1u) head = sum;
+    if ((later >> k) & 1u) *rp = sum;
+    if ((dm >> k) & 1u) {
+      sum = AT(0);
+      ++rp;
+      --vp;
+    }
+  }
+  // inclusive scan of the open runs; a lane that ends a row starts a new run
+  const bool hd = dm != 0u;
+  const uint32_t heads = __ballot_sync(0xffffffffu, hd);
+  if (lane == 0 && !hd) sum += carry;
+  const uint32_t upto = heads & (0xffffffffu >> (31 - lane));
+  const int dist = upto ? lane - (31 - __clz(upto)) : lane;   // lanes back to the run's start
+  uint32_t run = ~heads & ~1u;                        // lanes that continue a run
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    if (run == 0u) break;                             // no run is longer (the same in every lane)
+    const AT up = __shfl_up_sync(0xffffffffu, sum, o);
+    if (o <= dist) sum += up;
+    run &= run >> o;
+  }
+  // the run that reaches this lane's first row
+  const AT up = __shfl_up_sync(0xffffffffu, sum, 1);
+  if (hd) sy[y0] = head + (lane == 0 ? carry : up);
+  return __shfl_sync(0xffffffffu, sum, 31);
+}
+
+// The sum of a tile of one row: lanes take every 32nd nonzero (vp, left: from the lane's first).
+template <typename VT, typename XT, typename AT>
+__device__ __forceinline__ AT walk_row(const VT* vp, const XT (&xv)[kSigmaMax], int left) {
+  AT sum = AT(0);
+#pragma unroll
+  for (int k = 0; k < kSigmaMax; ++k) {
+    if (32 * k < left) {
+      if constexpr (!IsUnit<VT>::value) sum = mul_add(static_cast<AT>(widen(vp[32 * k])), static_cast<AT>(xv[k]), sum);
+      else sum += static_cast<AT>(xv[k]);
+    }
+  }
+  return warp_sum(sum);
+}
+
 // Boundary k of the units (c tiles each): the row open there.  Every distinct row of the
 // unit boundaries is written once, by its first boundary, from its FP64 accumulator.
 template <typename Epi>
@@ -337,58 +398,8 @@ __global__ void __launch_bounds__(kWalkThreads, CTAS)
       }
     }
     AT* const sy = sy_end - n_t;                     // the tile's row sums
-    if (!single) {
-      const uint32_t first = dm & (0u - dm);         // the lane's first down step
-      const uint32_t later = dm ^ first;
-      const VT* vp = sv + (vpad + xo);
-      AT* rp = sy + y0;
-      AT sum = AT(0), head = AT(0);
-#pragma unroll
-      for (int k = 0; k < kSigmaMax; ++k) {
-        if constexpr (kVals) {
-          const AT v = static_cast<AT>(widen(vp[k]));
-          if ((rm >> k) & 1u) sum = mul_add(v, static_cast<AT>(xv[k]), sum);
-        } else {
-          if ((rm >> k) & 1u) sum += static_cast<AT>(xv[k]);
-        }
-        if ((first >> k) & 1u) head = sum;
-        if ((later >> k) & 1u) *rp = sum;
-        if ((dm >> k) & 1u) {
-          sum = AT(0);
-          ++rp;
-          --vp;
-        }
-      }
-      // inclusive scan of the open runs; a lane that ends a row starts a new run
-      const bool hd = dm != 0u;
-      const uint32_t heads = __ballot_sync(0xffffffffu, hd);
-      if (lane == 0 && !hd) sum += carry;
-      const uint32_t upto = heads & (0xffffffffu >> (31 - lane));
-      const int dist = upto ? lane - (31 - __clz(upto)) : lane;   // lanes back to the run's start
-      uint32_t run = ~heads & ~1u;                    // lanes that continue a run
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        if (run == 0u) break;                         // no run is longer (the same in every lane)
-        const AT up = __shfl_up_sync(0xffffffffu, sum, o);
-        if (o <= dist) sum += up;
-        run &= run >> o;
-      }
-      // the run that reaches this lane's first row
-      const AT up = __shfl_up_sync(0xffffffffu, sum, 1);
-      if (hd) sy[y0] = head + (lane == 0 ? carry : up);
-      carry = __shfl_sync(0xffffffffu, sum, 31);
-    } else {
-      const VT* vp = sv + (vpad + lane);
-      AT sum = AT(0);
-#pragma unroll
-      for (int k = 0; k < kSigmaMax; ++k) {
-        if (lane + 32 * k < xe - xs) {
-          if constexpr (kVals) sum = mul_add(static_cast<AT>(widen(vp[32 * k])), static_cast<AT>(xv[k]), sum);
-          else sum += static_cast<AT>(xv[k]);
-        }
-      }
-      carry += warp_sum(sum);
-    }
+    if (!single) carry = walk_lanes<VT, XT, AT>(sv + (vpad + xo), xv, rm, dm, sy, y0, carry, lane);
+    else carry += walk_row<VT, XT, AT>(sv + (vpad + lane), xv, xe - xs - lane);
     __syncwarp();
 
     // ---- commit: the tile's rows; the unit's first row may have begun in another unit

@@ -114,3 +114,36 @@ def test_units_write_every_row_once(case, sigma, c):
     assert (writes == 1).all(), np.flatnonzero(writes != 1)[:10]
     ref, d = oracle.spmv(a.row_ptr, a.col, a.val, x)
     assert oracle.relative_errors(y, ref, d).max() <= 1e-12
+
+
+@pytest.mark.parametrize("sigma", [14, 5])
+@pytest.mark.parametrize("case", sorted(CASES))
+def test_tile_shares_add_up_to_the_rows(case, sigma):
+    """The one-launch PageRank stores, per tile, its share of its first row (if the row ends in
+    it) and of the row open at its end; the first tile that starts in a row adds them up."""
+    a = CASES[case]()
+    x = np.random.default_rng(1).random(a.n_cols)
+    t = oracle.build_tile(a.row_ptr, sigma)
+    T, n = t["tile_num"], a.n_rows
+    tx, rows = t["tile_x"].astype(np.int64), t["tile_y"].astype(np.int64) & ~MSB
+    prod = a.val * x[a.col]
+    y, writes = np.zeros(n), np.zeros(n, np.int64)
+    head, tail = np.full(T, np.nan), np.full(T, np.nan)
+    for i in range(T):
+        for r in range(rows[i], rows[i + 1]):
+            s = float(prod[max(tx[i], a.row_ptr[r]):a.row_ptr[r + 1]].sum())
+            if r == rows[i]:
+                head[i] = s
+            else:
+                y[r] = s
+                writes[r] += 1
+        last = rows[i + 1]
+        tail[i] = float(prod[max(tx[i], a.row_ptr[last]) if last < n else tx[i + 1]:tx[i + 1]].sum())
+    for i in range(T):
+        if np.searchsorted(rows, rows[i], side="left") == i:
+            span = int(np.searchsorted(rows, rows[i], side="right")) - i
+            y[rows[i]] = head[i + span - 1] + sum(tail[i + q - 1] for q in range(span) if i + q > 0)
+            writes[rows[i]] += 1
+    assert (writes == 1).all()
+    ref, d = oracle.spmv(a.row_ptr, a.col, a.val, x)
+    assert oracle.relative_errors(y, ref, d).max() <= 1e-12
