@@ -195,7 +195,8 @@ int persistent_grid(const void* kernel, int threads, size_t smem, size_t smem_ma
   size_t& lim = attr[std::make_pair(dev, kernel)];
   // a refused request (more shared memory than a CTA may have) is an answer, not an error
   // for later calls: the runtime's last-error state is cleared
-  if (smem_max > 48 * 1024 && lim < smem_max) {
+  // (the default limit of 48 KB counts the kernel's static shared memory, a few KB, too)
+  if (smem_max > 40 * 1024 && lim < smem_max) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max) !=
         cudaSuccess) {
       cudaGetLastError();
