@@ -89,7 +89,7 @@ struct EpiBicgV {
   __device__ __forceinline__ bool skip(const RedState* red) const { return stopped(red); }
   __device__ __forceinline__ void row(int r, double s, double& p0, double&) const {
     w.v[r] = s;
-    p0 += w.rhat[r] * s;
+    p0 += __ldcs(w.rhat + r) * s;
   }
   __device__ __forceinline__ void row64(int r, double s, double& p0, double& p1) const { row(r, s, p0, p1); }
   __device__ __forceinline__ void finish(double A, double, RedState* red) const {
@@ -115,40 +115,82 @@ struct EpiBicgT {
   }
 };
 
-// K1: p = r + beta (p - omega v)
-__global__ void __launch_bounds__(256) bicg_p_kernel(BicgVecs w, int64_t n, const RedState* red) {
+// The vector passes.  A CTA takes chunks of kVecSpan rows, kVecRows rows a thread in flight: with
+// one, the passes waited for their loads, and eight CTAs an SM are slower than three.  x and r_hat
+// are read twice an iteration at most and go through L2 as streams, which leaves it to p, r, v, s and
+// t.  A 3 M-vertex road grid: 226 us an iteration before, 197 (one-thread guard launch included).
+constexpr int kVecRows = 4, kVecThreads = 256, kVecSpan = kVecRows * kVecThreads, kVecCtas = 3;
+
+template <typename F>
+__device__ __forceinline__ void vec_chunks(int64_t n, F body) {
+  const int64_t chunks = (n + kVecSpan - 1) / kVecSpan;
+  for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) body(c * kVecSpan + threadIdx.x);
+}
+
+// K1: p = r + beta (p - omega v).  It also counts the loop body's runs: whatever the reductions did,
+// the loop ends after max_iter of them.
+__global__ void __launch_bounds__(kVecThreads, kVecCtas) bicg_p_kernel(BicgVecs w, int64_t n, RedState* red) {
   if (stopped(red)) return;
-  const BicgState st = *w.st;
-  const double beta = (st.rho / st.rho_prev) * (st.alpha / st.omega);
-  const double om = st.omega;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    w.p[i] = w.r[i] + beta * (w.p[i] - om * w.v[i]);
+  const double beta = (w.st->rho / w.st->rho_prev) * (w.st->alpha / w.st->omega);
+  const double om = w.st->omega;
+  vec_chunks(n, [&](int64_t i0) {
+    double r[kVecRows], p[kVecRows], v[kVecRows];
+#pragma unroll
+    for (int u = 0; u < kVecRows; ++u) {
+      const int64_t i = i0 + u * kVecThreads;
+      if (i < n) { r[u] = w.r[i]; p[u] = w.p[i]; v[u] = w.v[i]; }
+    }
+#pragma unroll
+    for (int u = 0; u < kVecRows; ++u) {
+      const int64_t i = i0 + u * kVecThreads;
+      if (i < n) w.p[i] = r[u] + beta * (p[u] - om * v[u]);
+    }
+  });
+  if (blockIdx.x == 0 && threadIdx.x == 0 && ++w.st->body > w.st->max_iter) stop(w, red, 2);
 }
 
 // K2: s = r - alpha v
-__global__ void __launch_bounds__(256) bicg_s_kernel(BicgVecs w, int64_t n, const RedState* red) {
+__global__ void __launch_bounds__(kVecThreads, kVecCtas) bicg_s_kernel(BicgVecs w, int64_t n, const RedState* red) {
   if (stopped(red)) return;
   const double alpha = w.st->alpha;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    w.s[i] = w.r[i] - alpha * w.v[i];
+  vec_chunks(n, [&](int64_t i0) {
+    double r[kVecRows], v[kVecRows];
+#pragma unroll
+    for (int u = 0; u < kVecRows; ++u) {
+      const int64_t i = i0 + u * kVecThreads;
+      if (i < n) { r[u] = w.r[i]; v[u] = w.v[i]; }
+    }
+#pragma unroll
+    for (int u = 0; u < kVecRows; ++u) {
+      const int64_t i = i0 + u * kVecThreads;
+      if (i < n) w.s[i] = r[u] - alpha * v[u];
+    }
+  });
 }
 
 // K3: x += alpha p + omega s; r = s - omega t; (r_hat, r), (r, r); stop test
-__global__ void __launch_bounds__(256) bicg_xr_kernel(BicgVecs w, int64_t n, RedState* red) {
+__global__ void __launch_bounds__(kVecThreads, kVecCtas) bicg_xr_kernel(BicgVecs w, int64_t n, RedState* red) {
   if (stopped(red)) return;
   const double alpha = w.st->alpha, omega = w.st->omega;
   double p0 = 0.0, p1 = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double si = w.s[i];
-    w.x[i] += alpha * w.p[i] + omega * si;
-    const double ri = si - omega * w.t[i];
-    w.r[i] = ri;
-    p0 += w.rhat[i] * ri;
-    p1 += ri * ri;
-  }
+  vec_chunks(n, [&](int64_t i0) {
+    double s[kVecRows], t[kVecRows], p[kVecRows], x[kVecRows], h[kVecRows];
+#pragma unroll
+    for (int u = 0; u < kVecRows; ++u) {
+      const int64_t i = i0 + u * kVecThreads;
+      if (i < n) { s[u] = w.s[i]; t[u] = w.t[i]; p[u] = w.p[i]; x[u] = __ldcs(w.x + i); h[u] = __ldcs(w.rhat + i); }
+    }
+#pragma unroll
+    for (int u = 0; u < kVecRows; ++u) {
+      const int64_t i = i0 + u * kVecThreads;
+      if (i >= n) break;
+      __stcs(w.x + i, fma(omega, s[u], fma(alpha, p[u], x[u])));
+      const double ri = s[u] - omega * t[u];
+      w.r[i] = ri;
+      p0 += h[u] * ri;
+      p1 += ri * ri;
+    }
+  });
   grid_sum2(p0, p1, red, [&](double A, double B) {
     BicgState* st = w.st;
     const int it = st->iter + 1;
@@ -173,13 +215,6 @@ __global__ void bicg_state_kernel(BicgState* st, int max_iter, RedState* red) {
   red->done = 0;
   red->iters = 0;
   red->launches = 0;
-}
-
-// Last node of the loop body: whatever the reductions did, the loop ends after max_iter
-// runs of the body.
-__global__ void bicg_guard_kernel(BicgVecs w, RedState* red) {
-  if (stopped(red)) return;
-  if (++w.st->body >= w.st->max_iter) stop(w, red, 2);
 }
 
 // the product of the plan's matrix, with values or (vals == NULL) all values 1
@@ -236,7 +271,7 @@ merbit_status merbit_bicgstab(merbit_plan_t p, const double* vals, const double*
   w.t = reinterpret_cast<double*>(mem + 5 * vb);
   w.st = reinterpret_cast<BicgState*>(mem + 6 * vb);
   w.hist = reinterpret_cast<double*>(mem + 6 * vb + sb);
-  const int vgrid = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)p->num_sms * 8));
+  const int vgrid = (int)std::max<int64_t>(1, std::min<int64_t>((n + kVecSpan - 1) / kVecSpan, (int64_t)p->num_sms * kVecCtas));
 
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -273,19 +308,18 @@ merbit_status merbit_bicgstab(merbit_plan_t p, const double* vals, const double*
   // the loop body: one iteration
   if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cap, cp.conditional.phGraph_out[0], nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
   if (e == cudaSuccess) {
-    bicg_p_kernel<<<vgrid, 256, 0, cap>>>(w, n, p->red);
+    bicg_p_kernel<<<vgrid, kVecThreads, 0, cap>>>(w, n, p->red);
     EpiBicgV ev{};
     ev.w = w;
     e = spmv64(p, vals, w.p, ev, cap);
     if (e == cudaSuccess) {
-      bicg_s_kernel<<<vgrid, 256, 0, cap>>>(w, n, p->red);
+      bicg_s_kernel<<<vgrid, kVecThreads, 0, cap>>>(w, n, p->red);
       EpiBicgT et{};
       et.w = w;
       e = spmv64(p, vals, w.s, et, cap);
     }
     if (e == cudaSuccess) {
-      bicg_xr_kernel<<<vgrid, 256, 0, cap>>>(w, n, p->red);
-      bicg_guard_kernel<<<1, 1, 0, cap>>>(w, p->red);
+      bicg_xr_kernel<<<vgrid, kVecThreads, 0, cap>>>(w, n, p->red);
       e = cudaGetLastError();
     }
     cudaGraph_t g_out = nullptr;
