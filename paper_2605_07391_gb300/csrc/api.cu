@@ -561,20 +561,21 @@ merbit_status merbit_ppr(merbit_plan_t p, const float* vals, const int32_t* seed
   if (merbit_status s = ensure_dangling(p, st)) return s;
   if (merbit_status s = ensure_hist(p, (size_t)max_iter, st)) return s;
   if (merbit_status s = ensure_spmm_acc(p, st)) return s;
-  // scratch: second iterate | seeds | D per column | 2k accumulators | last residuals
+  // scratch: second iterate | seeds | D per column | sets of 2k accumulators | last residuals
   const size_t xb = align256(sizeof(float) * (size_t)n * (size_t)k);
   const size_t sb = align256(sizeof(int32_t) * (size_t)k);
   const size_t db = align256(sizeof(double) * (size_t)k);
-  MB_TRY(grow(&p->scratch, &p->scratch_bytes, xb + sb + 4 * db, st));
+  const size_t rb = align256(sizeof(double) * ppr_sums(k));
+  MB_TRY(grow(&p->scratch, &p->scratch_bytes, xb + sb + 2 * db + rb, st));
   char* base = static_cast<char*>(p->scratch);
   float* x1 = reinterpret_cast<float*>(base);
   int32_t* seed_d = reinterpret_cast<int32_t*>(base + xb);
   double* d_cur = reinterpret_cast<double*>(base + xb + sb);
   double* rd = reinterpret_cast<double*>(base + xb + sb + db);
-  double* last_r = reinterpret_cast<double*>(base + xb + sb + 3 * db);
+  double* last_r = reinterpret_cast<double*>(base + xb + sb + db + rb);
   MB_TRY(cudaMemcpyAsync(seed_d, seeds, sizeof(int32_t) * (size_t)k, cudaMemcpyHostToDevice, st));
   MB_TRY(reset_device_state(p, st));
-  MB_TRY(cudaMemsetAsync(rd, 0, 2 * sizeof(double) * (size_t)k, st));
+  MB_TRY(cudaMemsetAsync(rd, 0, sizeof(double) * ppr_sums(k), st));
   MB_TRY(ppr_init(p, Pi, k, seed_d, d_cur, st));
   float* buf[2] = {Pi, x1};
   const int kBatch = 8;

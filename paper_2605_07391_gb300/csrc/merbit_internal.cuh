@@ -213,7 +213,8 @@ cudaError_t ppr_init(const merbit_plan_s* p, float* X, int64_t k, const int32_t*
                      double* d_cur, cudaStream_t st);
 // one update Y = alpha P^T X + (alpha D + 1 - alpha) e_seed for all k columns, then the
 // finish step (per-column residuals into last_r, D of Y into d_cur, hist[iter] = largest
-// residual, stop flag when it is below tol); rd: 2k zeroed FP64 accumulators (left zeroed)
+// residual, stop flag when it is below tol); rd: ppr_sums(k) zeroed FP64 accumulators (left zeroed)
+size_t ppr_sums(int64_t k);
 cudaError_t ppr_update(merbit_plan_s* p, const float* vals, const float* X, float* Y,
                        int64_t k, const int32_t* seed, double* d_cur, double* rd, double* last_r,
                        float alpha, double tol, int iter, double* hist, double* acc,

@@ -4,7 +4,7 @@
 //   1. the SpMM Y = alpha P^T X (one launch per column chunk, plus its finalize);
 //   2. a streaming pass over Y and X: the teleport and dangling mass alpha D_c + 1 - alpha
 //      added at each column's seed, and per column ||Y - X||_1 and the dangling mass of Y;
-//   3. a one-block finish: D for the next update, the residuals, the stop test.
+//   3. by the pass's last block: D for the next update, the residuals, the stop test.
 #include "spmm_kernel.cuh"
 
 namespace merbit {
@@ -23,28 +23,42 @@ __global__ void ppr_init_kernel(float* X, int64_t ldx, const int32_t* seed, int 
   }
 }
 
-// Step 2.  A block's threads cover rpb rows x (k / VW) column vectors of the row-major
-// arrays, so a thread keeps VW columns; rows advance by gridDim.x * rpb, four rows per
-// round with all their loads issued first.  Partial sums run in f32 over 16 rows and are
-// then added in FP64; the block's per-column totals are summed from a per-thread slot array.
-// rd[c] += ||Y_c - X_c||_1, rd[k + c] += sum over dangling r of Y[r, c].
+// Steps 2 and 3.  A block's threads cover rpb rows x (k / VW) column vectors of the row-major
+// arrays, so a thread keeps VW columns; rows advance by gridDim.x * rpb, two rows per
+// round with all their loads issued first; X is not read again and goes through L2 as a stream.  Partial sums run in f32 over 16 rows and are
+// then added in FP64; the block's per-column totals come from a per-thread slot array, in two
+// stages of at most 16 segments, and go to one of kPprSlots sets of accumulators (blocks that
+// finish together would queue for one set's cache line).
+// rd[slot][c] += ||Y_c - X_c||_1, rd[slot][k + c] += sum over dangling r of Y[r, c].
+// The block that arrives last adds the sets and clears them: D for the next update, the
+// per-column residuals, the largest residual into the history, the stop test.
+// The pass reads 8 n k bytes and is bound by them and by 8 FP64 adds and conversions per thread
+// and 16 rows.  One whole update, n = 2^20, 17 M nonzeros, k = 8:
+// 115.2 us an update before (two blocks of four rows in flight an SM, 128 rows added up one
+// after the other at a block's end, a one-block launch for the finish), 110.9; k = 32: 335, 318.
+constexpr int kPprSlots = 16;
+constexpr int kPprSegs = 16;
+
 template <int VW>
-__global__ void __launch_bounds__(VW == 4 ? 256 : 1024)     // k <= 1024: k / 4 <= 256 vectors
+__global__ void __launch_bounds__(VW == 4 ? 256 : 1024, VW == 4 ? 4 : 1)   // k <= 1024: k / 4 <= 256 vectors
     ppr_stream_kernel(float* __restrict__ Y, const float* __restrict__ X, int64_t n, int k,
-                      const int32_t* __restrict__ seed, const double* __restrict__ d_cur,
-                      const uint32_t* __restrict__ dang, float alpha, double* rd,
-                      const RedState* red) {
+                      const int32_t* __restrict__ seed, double* d_cur,
+                      const uint32_t* __restrict__ dang, float alpha, double* rd, double* last_r,
+                      double tol, int iter, double* hist, RedState* red) {
   using V = SpmmVec<VW>;
   using VT = typename V::T;
-  constexpr int R = 4;                           // rows per round
-  extern __shared__ double sred[];               // [rpb * kv][VW][2] partials of the threads
+  constexpr int R = 2;                           // rows per round
+  extern __shared__ double sred[];               // [rpb * kv][VW][2] partials of the threads, then
+  double* const sseg = sred + 2 * VW * blockDim.x;   // [segs][2k] of the segments
+  __shared__ unsigned long long smax;
+  __shared__ int last;
   if (*reinterpret_cast<const volatile int*>(&red->done)) return;
   const int kv = k / VW;
   const int rpb = blockDim.x / kv;
   const int t = threadIdx.x;
   if (t < rpb * kv) {
     const int c = (t % kv) * VW;
-    int64_t s[VW];
+    int s[VW];
     float tel[VW];
     double res[VW], dm[VW];
 #pragma unroll
@@ -73,7 +87,7 @@ __global__ void __launch_bounds__(VW == 4 ? 256 : 1024)     // k <= 1024: k / 4 
           if (ru < n) {
             const size_t e = (size_t)ru * k + c;
             yv[u] = V::load_plain(Y + e);
-            xv[u] = V::load(X + e);
+            xv[u] = __ldcs(reinterpret_cast<const VT*>(X + e));
             dg[u] = is_dangling(dang, (int)ru);
           }
         }
@@ -111,39 +125,59 @@ __global__ void __launch_bounds__(VW == 4 ? 256 : 1024)     // k <= 1024: k / 4 
     }
   }
   __syncthreads();
-  for (int i = t; i < 2 * k; i += blockDim.x) {
+  const int items = 2 * k;
+  const int segs = min(min((int)blockDim.x / items, rpb), kPprSegs);
+  double* const slot = rd + (size_t)(blockIdx.x % kPprSlots) * items;
+  auto total = [&](int i, int first, int every) {
     const int part = i / k, col = i % k, cv = col / VW, j = col % VW;
     double tot = 0.0;
-    for (int rho = 0; rho < rpb; ++rho) tot += sred[((rho * kv + cv) * VW + j) * 2 + part];
-    atomicAdd(rd + i, tot);
+    for (int rho = first; rho < rpb; rho += every) tot += sred[((rho * kv + cv) * VW + j) * 2 + part];
+    return tot;
+  };
+  if (segs > 1) {
+    if (t < items * segs) sseg[t] = total(t % items, t / items, segs);
+    __syncthreads();
+    if (t < items) {
+      double tot = 0.0;
+      for (int q = 0; q < segs; ++q) tot += sseg[q * items + t];
+      atomicAdd(slot + t, tot);
+    }
+  } else {
+    for (int i = t; i < items; i += blockDim.x) atomicAdd(slot + i, total(i, 0, 1));
   }
-}
-
-// Step 3: D for the next update, the per-column residuals, the largest residual into the
-// history, the stop test, and the accumulators cleared.
-__global__ void ppr_finish_kernel(double* rd, double* d_cur, double* last_r, int k, double tol,
-                                  int iter, double* hist, RedState* red) {
-  __shared__ double smax[256];
-  if (*reinterpret_cast<const volatile int*>(&red->done)) return;
+  __threadfence();
+  __syncthreads();
+  if (t == 0) {
+    smax = 0ull;
+    last = atomicAdd(&red->arrive, 1u) + 1 == gridDim.x;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   double m = 0.0;
-  for (int c = threadIdx.x; c < k; c += blockDim.x) {
-    const double r = rd[c];
+  for (int c = t; c < k; c += blockDim.x) {
+    double r = 0.0, dm = 0.0;
+#pragma unroll 4
+    for (int q = 0; q < kPprSlots; ++q) {
+      double* a = rd + (size_t)q * items + c;
+      r += __ldcg(a);
+      dm += __ldcg(a + k);
+      __stcg(a, 0.0);
+      __stcg(a + k, 0.0);
+    }
     last_r[c] = r;
-    d_cur[c] = rd[k + c];
-    rd[c] = 0.0;
-    rd[k + c] = 0.0;
+    d_cur[c] = dm;
     m = fmax(m, r);
   }
-  smax[threadIdx.x] = m;
+  // the largest of the threads' maxima, none negative or NaN: their bits compare as integers
+  if (t < k) atomicMax(&smax, (unsigned long long)__double_as_longlong(m));
   __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + h]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    hist[iter] = smax[0];
+  if (t == 0) {
+    m = __longlong_as_double((long long)smax);
+    red->arrive = 0u;
+    hist[iter] = m;
     ++red->launches;
-    if (tol > 0.0 && smax[0] < tol) {
+    if (tol > 0.0 && m < tol) {
       red->iters = iter + 1;
       red->done = 1;
     }
@@ -151,6 +185,8 @@ __global__ void ppr_finish_kernel(double* rd, double* d_cur, double* last_r, int
 }
 
 }  // namespace
+
+size_t ppr_sums(int64_t k) { return (size_t)kPprSlots * 2 * (size_t)k; }
 
 cudaError_t ppr_init(const merbit_plan_s* p, float* X, int64_t k, const int32_t* seed,
                      double* d_cur, cudaStream_t st) {
@@ -173,17 +209,14 @@ cudaError_t ppr_update(merbit_plan_s* p, const float* vals, const float* X, floa
   const int rpb = kv <= kStreamThreads ? kStreamThreads / kv : 1;
   const int threads = rpb * kv;
   const int64_t blocks_needed = (p->n_rows + rpb - 1) / rpb;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks_needed, (int64_t)p->num_sms * 2));
-  const size_t sm = 2 * sizeof(double) * (size_t)threads * (vec ? 4 : 1);
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(blocks_needed, (int64_t)p->num_sms * (threads <= 256 ? 4 : 2)));
+  const size_t sm = sizeof(double) * (size_t)threads * (vec ? 9 : 3);
   if (vec)
     ppr_stream_kernel<4><<<grid, threads, sm, st>>>(Y, X, p->n_rows, (int)k, seed, d_cur,
-                                                    p->dangling_bits, alpha, rd, p->red);
+                                                    p->dangling_bits, alpha, rd, last_r, tol, iter, hist, p->red);
   else
     ppr_stream_kernel<1><<<grid, threads, sm, st>>>(Y, X, p->n_rows, (int)k, seed, d_cur,
-                                                    p->dangling_bits, alpha, rd, p->red);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  ppr_finish_kernel<<<1, 256, 0, st>>>(rd, d_cur, last_r, (int)k, tol, iter, hist, p->red);
+                                                    p->dangling_bits, alpha, rd, last_r, tol, iter, hist, p->red);
   return cudaGetLastError();
 }
 
