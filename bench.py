@@ -500,7 +500,7 @@ def run_many_graphs(args, dev, stream) -> dict:
     # sigma x block kernel by measurement (batches keep 8 tiles per block and 32-bit
     # descriptors; the block size is listed for completeness)
     tune, times = mb.autotune(rp, col, vals, sigmas=(14, 12, 10, 7), blocks=(8,),
-                              kernels=("classic", "split", "split2"), hots=(0,), reps=3, stream=stream)
+                              kernels=("auto", "classic", "split", "split2"), hots=(0,), reps=3, stream=stream)
     best = tune["sigma"]
     res["autotune"] = {"best": tune, "ms_per_spmv": {f"s{k[0]}_W{k[1]}_{k[2]}": v for k, v in times.items()}}
     torch.cuda.synchronize(dev)
@@ -875,8 +875,8 @@ def main():
                         "traffic_bytes_per_nnz": traffic / a.nnz if traffic else None,
                         "algorithmic_bytes_per_launch": alg_bytes,
                         "bytes_per_nnz": alg_bytes / a.nnz, "parts": alg_parts,
-                        "kernel": "merbit_spmv_split_kernel<float,float,float,EpiPlain> (the default block "
-                                  "kernel for f32 values) + merbit_finalize_kernel",
+                        "kernel": "merbit_spmv_walk_kernel<float,float,float,EpiPlain> (the automatic "
+                                  "choice without a hot-column table) + merbit_walk_finalize_kernel",
                         "mean_launch_ms": mean_launch_ms,
                         "median_launch_ms": statistics.median(launch_ms)},
            "plan_ms": plan_ms, "gen_s": gen_s,
