@@ -30,25 +30,32 @@
 // f64: this GPU has two FP64 lanes per SM and clock, so a warp instruction of FP64 holds the
 // SM's pipe for 16 cycles; the fused multiply-add halves the work per nonzero (the split
 // kernel multiplies, stores and adds) and row ends cost one add instead of two atomics.
-// R-MAT scale 22 with 30 % empty rows, f64: 0.336 -> 0.215 ms (pipe 56 % busy).
+// R-MAT scale 22 with 30 % empty rows, f64: 0.336 -> 0.203 ms (pipe 56 % busy at 0.215).
 #pragma once
 
 namespace merbit {
 
-// Elements of a warp's buffers: a tile's 32 sigma steps, up to 7 elements of alignment
-// before its first nonzero, and the lane walk's reads past a lane's last product (13).
+// Elements of a tile's buffer in the kernels that share the walk: its 32 sigma steps, up to 7
+// elements of alignment before its first nonzero, and the walk's reads past a lane's last product.
 __host__ __device__ constexpr int walk_cap(int sigma) { return kOmega * sigma + 32; }
 
-// The value buffer also receives the tile's row sums, at its end: the nonzeros and rows of a
-// tile are at most 32 sigma together.
+// This kernel's buffers are as small as the copies allow.  Values: the tile's nonzeros with less
+// than 16 bytes before and after them (the copy's boundaries), and at the buffer's end the tile's
+// row sums; nonzeros and rows are at most 32 sigma together.  Columns: the nonzeros with less than
+// 16 bytes on either side.  What a lane reads past its last product (13 elements, never used)
+// lies in the buffer behind, or in the CTA's kWalkTail bytes.  That leaves three f64 CTAs at
+// sigma 14 (131 KB with the system's share) the next smaller carveout of shared memory, and L1 32
+// KB more than with 32 elements of slack in each buffer (139 KB): R-MAT scale 24, f64, 1.324 ms
+// and 1.155; scale 22 with 30 % empty rows 0.214 and 0.203.
 template <typename VT, typename AT>
 __host__ __device__ constexpr size_t walk_val_bytes(int sigma) {
-  return (sizeof(VT) > sizeof(AT) ? sizeof(VT) : sizeof(AT)) * (size_t)walk_cap(sigma);
+  return (sizeof(VT) > sizeof(AT) ? sizeof(VT) : sizeof(AT)) * (size_t)(kOmega * sigma) + 32;
 }
 template <typename VT, typename AT>
 __host__ __device__ constexpr size_t walk_warp_bytes(int sigma) {
-  return walk_val_bytes<VT, AT>(sigma) + sizeof(int32_t) * (size_t)walk_cap(sigma);
+  return walk_val_bytes<VT, AT>(sigma) + sizeof(int32_t) * (size_t)(kOmega * sigma) + 32;
 }
+constexpr size_t kWalkTail = 128;
 
 __device__ __forceinline__ void gather_if(float& v, const float* p, uint32_t pred, uint64_t pol) {
   asm volatile(
@@ -493,8 +500,8 @@ template <typename VT, typename XT, typename AT, typename Epi>
 cudaError_t launch_walk(const merbit_plan_s* p, const VT* vals, const XT* x, const Epi& epi, cudaStream_t st) {
   auto kern = merbit_spmv_walk_kernel<VT, XT, AT, Epi, kWalkCtas<AT>>;
   const void* kp = reinterpret_cast<const void*>(kern);
-  const size_t smem = kWalkWarps * walk_warp_bytes<VT, AT>(p->sigma);
-  int grid = persistent_grid(kp, kWalkThreads, smem, kWalkWarps * walk_warp_bytes<VT, AT>(kSigmaMax), p->num_sms);
+  const size_t smem = kWalkWarps * walk_warp_bytes<VT, AT>(p->sigma) + kWalkTail;
+  int grid = persistent_grid(kp, kWalkThreads, smem, kWalkWarps * walk_warp_bytes<VT, AT>(kSigmaMax) + kWalkTail, p->num_sms);
   if (grid <= 0) return cudaErrorInvalidConfiguration;
   Geometry g = p->geom();
   g.unit = walk_unit(p->tile_num, (int64_t)grid * kWalkWarps, p->tiles_per_block);
