@@ -41,6 +41,7 @@ WORKLOADS = {
 }
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "spmv_f32_rmat24_traffic.txt")
 KERNEL_SOURCES = ["paper_2605_07391_gb300/csrc/spmv_kernel.cuh",
+                  "paper_2605_07391_gb300/csrc/spmv_walk_kernel.cuh",
                   "paper_2605_07391_gb300/csrc/spmv_f32.cu",
                   "paper_2605_07391_gb300/csrc/merbit_internal.cuh"]
 

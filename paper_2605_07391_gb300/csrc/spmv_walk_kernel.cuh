@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kWalkThreads, CTAS)
 
 // Resident CTAs per SM: 32 warps for 4-byte sums (R-MAT scale 24: 0.929 ms, 24 warps 0.952,
 // 16 warps 1.012), 24 for 8-byte ones, whose buffers (5.8 KB a warp) would leave L1 too
-// little at 32 (R-MAT scale 22 with 30 % empty rows: 0.216 ms; 32 warps 0.261, 16 warps 0.224).
+// little at 32 (R-MAT scale 22 with 30 % empty rows, with 46 KB a CTA: 0.216 ms; 32 warps 0.261, 16 warps 0.224).
 template <typename AT>
 constexpr int kWalkCtas = sizeof(AT) == 8 ? 3 : 4;
 
