@@ -60,14 +60,8 @@ void free_plan(merbit_plan_s* p) {
   if (!p) return;
   host_async_release(p);
   free_hot_table(p);
-  cudaFree(p->block);
-  cudaFree(p->dangling_bits);
-  cudaFree(p->scratch);
-  cudaFree(p->hist);
-  cudaFree(p->x_stage);
-  cudaFree(p->y_stage);
-  cudaFree(p->spmm_acc);
-  cudaFree(p->spmm_pack);
+  dev_free(p->device, {p->block, p->dangling_bits, p->scratch, p->hist, p->x_stage, p->y_stage, p->spmm_acc,
+                       p->spmm_pack});
   if (p->host_pinned) cudaFreeHost(p->host_pinned);
   delete p;
 }
@@ -335,11 +329,7 @@ merbit_status merbit_plan_ex(const int32_t* row_ptr, const int32_t* col_idx, int
   }
 
   merbit_plan_s* p = new merbit_plan_s();
-  auto bail = [&](merbit_status s) {
-    cudaDeviceSynchronize();
-    free_plan(p);
-    return s;
-  };
+  auto bail = [&](merbit_status s) { free_plan(p); return s; };
   cudaGetDevice(&p->device);
   cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device);
   p->n_rows = n_rows;
@@ -402,8 +392,6 @@ merbit_status merbit_plan(const int32_t* row_ptr, const int32_t* col_idx, int64_
 }
 
 void merbit_plan_destroy(merbit_plan_t plan) {
-  if (!plan) return;
-  cudaDeviceSynchronize();
   free_plan(plan);
 }
 

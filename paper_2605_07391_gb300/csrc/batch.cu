@@ -465,20 +465,9 @@ void free_batch(merbit_batch_s* b) {
   if (!b) return;
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
+  dev_free(b->plan->device, {b->off, b->inv_n, b->dang0, b->D, b->conv, b->acc, b->last_r, b->bs, b->blist, b->bcount,
+                             b->bflags, b->ccount, b->x1});
   merbit_plan_destroy(b->plan);
-  cudaFree(b->off);
-  cudaFree(b->inv_n);
-  cudaFree(b->dang0);
-  cudaFree(b->D);
-  cudaFree(b->conv);
-  cudaFree(b->acc);
-  cudaFree(b->last_r);
-  cudaFree(b->bs);
-  cudaFree(b->blist);
-  cudaFree(b->bcount);
-  cudaFree(b->bflags);
-  cudaFree(b->ccount);
-  cudaFree(b->x1);
   delete b;
 }
 
@@ -650,10 +639,11 @@ merbit_status merbit_batch_plan(const int32_t* row_ptr, const int32_t* col_idx, 
   std::vector<double> d0(G);
   for (size_t g = 0; g < G; ++g) d0[g] = (double)cnt_h[g] * inv_n[g];
   if (e == cudaSuccess) e = cudaMemcpy(b->dang0, d0.data(), sizeof(double) * G, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) cudaDeviceSynchronize();   // nothing may use the blocks that go
-  cudaFree(cnt);
-  cudaFree(err);
-  if (e != cudaSuccess) {
+  if (e == cudaSuccess) {
+    cudaFree(cnt);
+    cudaFree(err);
+  } else {
+    dev_free(p->device, {cnt, err});
     free_batch(b);
     return bfail(e == cudaErrorMemoryAllocation ? MERBIT_ENOMEM : MERBIT_ECUDA, "merbit_batch_plan: %s",
                  cudaGetErrorString(e));

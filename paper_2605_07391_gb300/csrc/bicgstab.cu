@@ -338,8 +338,8 @@ merbit_status merbit_bicgstab(merbit_plan_t p, const double* vals, const double*
   if (exec) cudaGraphExecDestroy(exec);
   if (graph) cudaGraphDestroy(graph);
   if (cap) cudaStreamDestroy(cap);
-  if (e != cudaSuccess) cudaDeviceSynchronize();   // nothing may use the block that goes
-  cudaFree(mem);
+  if (e == cudaSuccess) cudaFree(mem);
+  else dev_free(p->device, {mem});
   if (e != cudaSuccess) {
     char msg[256];
     std::snprintf(msg, sizeof(msg), "BiCGSTAB: %s", cudaGetErrorString(e));

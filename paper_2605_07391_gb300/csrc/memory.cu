@@ -42,8 +42,8 @@ cudaMemPool_t pool_of(int dev) {
 }  // namespace
 
 // The block may be used by work queued on `st` from here on, and by any stream once `st` has been
-// synchronised.  It is freed by cudaFree, which does not wait for work that still uses a block of
-// the pool: callers synchronise before.  A stream that is being captured gets cudaMalloc (and its
+// synchronised.  cudaFree does not wait for work that still uses a block of the pool: blocks that
+// any stream may be using go through dev_free.  A stream that is being captured gets cudaMalloc (and its
 // refusal): a pool allocation would become part of the graph.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
   *p = nullptr;
@@ -60,6 +60,27 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
     cudaMemPoolTrimTo(pool, 0);
   }
   return cudaMalloc(p, bytes ? bytes : 1);
+}
+
+cudaError_t device_wait(int device) {
+  int current = device;
+  cudaGetDevice(&current);
+  if (current != device) cudaSetDevice(device);
+  const cudaError_t e = cudaDeviceSynchronize();
+  if (current != device) cudaSetDevice(current);
+  return e;
+}
+
+// Objects are destroyed from any thread, with any device current (a finaliser, say): the wait is
+// for the device that holds the blocks.  Blocks that could not be waited for are left allocated
+// rather than handed out again under running work.
+void dev_free(int device, std::initializer_list<void*> blocks) {
+  if (device_wait(device) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  for (void* b : blocks)
+    if (b) cudaFree(b);
 }
 
 }  // namespace merbit

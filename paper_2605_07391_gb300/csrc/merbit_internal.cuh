@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "merbit.h"
 
 namespace merbit {
@@ -180,9 +182,15 @@ struct SweepParams {
   double eta;                   // inner stop: sweep size <= eta * ||r||_1
 };
 
-// A block of device memory from the library's pool (memory.cu); freed by cudaFree after the work
-// that uses it has been waited for.
+// A block of device memory from the library's pool (memory.cu); freed by dev_free, or by cudaFree
+// after the work that uses it has been waited for.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
+
+// Waits for all work of `device`, whichever device is current.
+cudaError_t device_wait(int device);
+
+// Frees blocks of `device` (null ones are skipped) after device_wait.
+void dev_free(int device, std::initializer_list<void*> blocks);
 
 // ---- launchers (one translation unit per value type) ----
 cudaError_t spmv_plain_f32(const merbit_plan_s* p, const float* vals, const float* x, float* y,

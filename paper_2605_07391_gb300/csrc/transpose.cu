@@ -434,8 +434,7 @@ cudaError_t build_transpose(merbit_transpose_s* t, const int32_t* row_ptr, const
 
 void free_transpose(merbit_transpose_s* t) {
   if (!t) return;
-  cudaDeviceSynchronize();   // work that reads the arrays
-  cudaFree(t->row_ptr_t);    // the three arrays' block
+  dev_free(t->device, {t->row_ptr_t});    // the three arrays' block
   delete t;
 }
 
