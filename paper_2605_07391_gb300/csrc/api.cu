@@ -58,6 +58,7 @@ size_t dtype_size(merbit_dtype d) {
 
 void free_plan(merbit_plan_s* p) {
   if (!p) return;
+  const RelaxedCalls relaxed;
   host_async_release(p);
   free_hot_table(p);
   dev_free(p->device, {p->block, p->dangling_bits, p->scratch, p->hist, p->x_stage, p->y_stage, p->spmm_acc,
@@ -69,8 +70,9 @@ void free_plan(merbit_plan_s* p) {
 cudaError_t grow(void** buf, size_t* cap, size_t need, cudaStream_t st) {
   if (*cap >= need) return cudaSuccess;
   if (*buf) {
-    cudaDeviceSynchronize();   // earlier calls may still use it
-    cudaFree(*buf);
+    int device = 0;
+    cudaGetDevice(&device);
+    dev_free(device, {*buf});   // earlier calls may still use it
   }
   *buf = nullptr;
   *cap = 0;

@@ -186,6 +186,13 @@ struct SweepParams {
 // after the work that uses it has been waited for.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
 
+// While one lives, unsafe calls (cudaMalloc, cudaFree) of this thread leave the captures of any thread alone.
+struct RelaxedCalls {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCalls() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Waits for all work of `device`, whichever device is current.
 cudaError_t device_wait(int device);
 

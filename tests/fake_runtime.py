@@ -1,6 +1,5 @@
 """The library linked against tests/fake_cudart.cpp, for tests of its host side without a GPU."""
 import ctypes
-import glob
 import os
 import shutil
 import subprocess
@@ -15,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 def library(folder):
     """The library's own objects with the stand-in runtime; calls it does not define return 0."""
     b.build()
-    objs = sorted(glob.glob(os.path.join(b.BUILD, "*.o")))
+    objs = [os.path.join(b.BUILD, os.path.basename(s)[:-3] + ".o") for s in b._sources()]
     nvcc = b._nvcc()
     inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
     cxx = shutil.which("g++")
