@@ -81,15 +81,6 @@ cudaError_t grow(void** buf, size_t* cap, size_t need, cudaStream_t st) {
   return e;
 }
 
-cudaError_t reset_device_state(merbit_plan_s* p, cudaStream_t st) {
-  // the state and the block and tile accumulators lie one behind the other
-  char* const end = reinterpret_cast<char*>(p->tile_acc + (p->tile_num + 1));
-  cudaError_t e = cudaMemsetAsync(p->red, 0, (size_t)(end - reinterpret_cast<char*>(p->red)), st);
-  if (e == cudaSuccess && p->spmm_acc)
-    e = cudaMemsetAsync(p->spmm_acc, 0, sizeof(double) * 32 * (size_t)spmm_acc_sets(p), st);
-  return e;
-}
-
 // err, done, iters of the plan's RedState, read through pinned memory.
 struct StateWord { int err, done, iters, inner_done, launches; };
 
@@ -283,6 +274,15 @@ merbit_status ensure_spmm_acc(merbit_plan_s* p, cudaStream_t st) {
 namespace merbit {
 void set_last_error(const char* msg) {
   std::snprintf(g_err, sizeof(g_err), "%s", msg);
+}
+
+cudaError_t reset_device_state(merbit_plan_s* p, cudaStream_t st) {
+  // the state and the block and tile accumulators lie one behind the other
+  char* const end = reinterpret_cast<char*>(p->tile_acc + (p->tile_num + 1));
+  cudaError_t e = cudaMemsetAsync(p->red, 0, (size_t)(end - reinterpret_cast<char*>(p->red)), st);
+  if (e == cudaSuccess && p->spmm_acc)
+    e = cudaMemsetAsync(p->spmm_acc, 0, sizeof(double) * 32 * (size_t)spmm_acc_sets(p), st);
+  return e;
 }
 }  // namespace merbit
 

@@ -346,7 +346,7 @@ merbit_status merbit_bicgstab(merbit_plan_t p, const double* vals, const double*
     return bfail2(MERBIT_ECUDA, msg);
   }
   if (err) {
-    cudaMemsetAsync(p->red, 0, sizeof(RedState), st);
+    reset_device_state(p, st);
     cudaStreamSynchronize(st);
     return bfail2(MERBIT_EDEVICE, "a kernel reported an error");
   }

@@ -199,6 +199,10 @@ cudaError_t device_wait(int device);
 // Frees blocks of `device` (null ones are skipped) after device_wait.
 void dev_free(int device, std::initializer_list<void*> blocks);
 
+// Clears the plan's reduction state and error bits, and every accumulator of rows between units and
+// blocks (a kernel that gave up may have left sums there).
+cudaError_t reset_device_state(merbit_plan_s* p, cudaStream_t st);
+
 // ---- launchers (one translation unit per value type) ----
 cudaError_t spmv_plain_f32(const merbit_plan_s* p, const float* vals, const float* x, float* y,
                            cudaStream_t st);

@@ -18,6 +18,8 @@ struct Block { int dev; size_t bytes; bool pool; };
 std::map<void*, Block> g_blocks;
 int g_dev = 0, g_busy[2] = {0, 0}, g_violations = 0, g_capturing = 0, g_broken = 0, g_mallocs = 0;
 cudaStreamCaptureMode g_mode = cudaStreamCaptureModeGlobal;
+void* g_set = nullptr;      // the first range cleared since fake_reset
+size_t g_set_bytes = 0;
 size_t g_used = 0, g_idle = 0, g_limit = ~size_t(0) >> 1;
 
 cudaError_t unsafe_call() {
@@ -39,6 +41,7 @@ void fake_reset() {
   g_mode = cudaStreamCaptureModeGlobal;
   g_limit = ~size_t(0) >> 1;
   g_idle = 0;
+  g_set = nullptr;
 }
 void fake_busy(int dev, int busy) { g_busy[dev] = busy; }
 void fake_capture(int on) { g_capturing = on; }
@@ -47,6 +50,7 @@ int fake_violations() { return g_violations; }
 int fake_broken() { return g_broken; }
 int fake_mallocs() { return g_mallocs; }
 int fake_device() { return g_dev; }
+void* fake_first_set(size_t* bytes) { *bytes = g_set_bytes; return g_set; }
 size_t fake_used() { return g_used; }
 size_t fake_idle() { return g_idle; }
 
@@ -100,7 +104,17 @@ cudaError_t cudaMallocHost(void** p, size_t n) { *p = std::calloc(1, n); return 
 cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
+  if (!g_set) g_set = d, g_set_bytes = n;
+  std::memset(d, v, n);
+  return cudaSuccess;
+}
+cudaError_t cudaGraphAddNode(cudaGraphNode_t*, cudaGraph_t, const cudaGraphNode_t*, const cudaGraphEdgeData*, size_t,
+                             cudaGraphNodeParams* params) {
+  static cudaGraph_t body[1];
+  if (params->type == cudaGraphNodeTypeConditional) params->conditional.phGraph_out = body;
+  return cudaSuccess;
+}
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
   *v = a == cudaDevAttrMultiProcessorCount ? 4 : a == cudaDevAttrMaxSharedMemoryPerBlockOptin ? 227 << 10
        : a == cudaDevAttrMaxSharedMemoryPerMultiprocessor ? 228 << 10 : 1;

@@ -34,6 +34,7 @@ def library(folder):
     subprocess.run([cxx, "-shared", "-Wl,-Bsymbolic", "-o", path, *objs, fake, stubs + ".o"], check=True)
     lib = ctypes.CDLL(path)
     lib.fake_used.restype = lib.fake_idle.restype = ctypes.c_size_t
+    lib.fake_first_set.restype = ctypes.c_void_p
     lib.fake_limit.argtypes = [ctypes.c_size_t]
     lib.merbit_last_error.restype = ctypes.c_char_p
     return lib

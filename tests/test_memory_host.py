@@ -1,4 +1,7 @@
 """Host-side rules of the library's device memory, against a stand-in CUDA runtime (no GPU)."""
+import ctypes
+
+import numpy as np
 import pytest
 
 from tests import fake_runtime as fr
@@ -32,3 +35,29 @@ def test_destroy_during_a_capture(lib, kind):
     lib.fake_capture(0)
     assert lib.fake_violations() == 0, "memory went back to the pool under running work"
     assert not lib.fake_broken(), "the capture was broken"
+
+
+@pytest.mark.parametrize("kind", ["bicgstab"])
+def test_state_is_clear_after_a_give_up(lib, kind):
+    """A kernel that gave up may leave sums in the accumulators between units, not the error bit
+    alone: both are cleared before the error is reported."""
+    lib.fake_reset()
+    m = fr.Pattern(lib)
+    h = m.batch() if kind == "batch" else m.plan()
+    size = ctypes.c_size_t()
+    at = lib.fake_first_set(ctypes.byref(size))    # the new plan's state and accumulators
+    state = np.ctypeslib.as_array((ctypes.c_ubyte * size.value).from_address(at))
+    state[:] = 0xFF
+    v = np.zeros(m.nnz + 2)
+    v = v[(-v.ctypes.data // 8) % 2:][:m.nnz]      # values on a 16-byte boundary
+    b, x = np.zeros(m.n), np.zeros(m.n)
+    vp, f64 = ctypes.c_void_p, ctypes.c_double
+    if kind == "batch":
+        st = lib.merbit_batch_pagerank(h, 1, vp(v.ctypes.data), f64(0.85), f64(0.0), 2, vp(x.ctypes.data), None, None,
+                                       None, None)
+    else:
+        st = lib.merbit_bicgstab(h, vp(v.ctypes.data), vp(b.ctypes.data), vp(x.ctypes.data), f64(0.0), 2, None, None,
+                                 None, None, None)
+    assert st == 6, lib.merbit_last_error()
+    assert not state.any()
+    getattr(lib, "merbit_batch_destroy" if kind == "batch" else "merbit_plan_destroy")(h)
