@@ -721,7 +721,7 @@ merbit_status merbit_batch_pagerank(merbit_batch_t b, merbit_dtype dtype, const 
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return bfail(MERBIT_ECUDA, "batched solve: %s", cudaGetErrorString(e));
   if (err) {
-    cudaMemsetAsync(b->plan->red, 0, sizeof(RedState), st);
+    reset_device_state(b->plan, st);
     cudaStreamSynchronize(st);
     return bfail(MERBIT_EDEVICE, "a kernel reported error bits 0x%x", err);
   }

@@ -37,7 +37,7 @@ def test_destroy_during_a_capture(lib, kind):
     assert not lib.fake_broken(), "the capture was broken"
 
 
-@pytest.mark.parametrize("kind", ["bicgstab"])
+@pytest.mark.parametrize("kind", ["bicgstab", "batch"])
 def test_state_is_clear_after_a_give_up(lib, kind):
     """A kernel that gave up may leave sums in the accumulators between units, not the error bit
     alone: both are cleared before the error is reported."""
