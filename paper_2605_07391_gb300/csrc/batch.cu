@@ -450,6 +450,7 @@ struct merbit_batch_s {
   cudaGraphExec_t exec = nullptr;
   merbit_dtype dt = MERBIT_F64;
   int spmv_kernel = -1;
+  uint32_t wait_limit = 0;             // the plan's, recorded in the kernels' arguments
   const int32_t* hot_list = nullptr;   // the plan's hot-column table when recorded
   const int32_t* col_hot = nullptr;
   int hot_n = -1;
@@ -673,7 +674,7 @@ merbit_status merbit_batch_pagerank(merbit_batch_t b, merbit_dtype dtype, const 
   const bool same = b->exec && b->dt == dtype && b->vals == vals && b->pi == pi && b->alpha == alpha &&
                     b->tol == tol && b->max_iter == max_iter && b->spmv_kernel == b->plan->spmv_kernel &&
                     b->hot_list == b->plan->hot_list && b->col_hot == b->plan->col_hot &&
-                    b->hot_n == b->plan->hot_n;
+                    b->hot_n == b->plan->hot_n && b->wait_limit == b->plan->wait_limit;
   if (!same) {
     if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
     if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
@@ -708,6 +709,7 @@ merbit_status merbit_batch_pagerank(merbit_batch_t b, merbit_dtype dtype, const 
     b->hot_list = b->plan->hot_list;
     b->col_hot = b->plan->col_hot;
     b->hot_n = b->plan->hot_n;
+    b->wait_limit = b->plan->wait_limit;
   }
   e = cudaGraphLaunch(b->exec, st);
   std::vector<int> conv((size_t)b->G);
