@@ -118,7 +118,7 @@ __global__ void pr_state_init_kernel(double* hist, double d0, RedState* red) {
   red->iters = 0;
   red->inner_done = 0;
   red->launches = 0;
-  red->bar = 0u;
+  red->bar = kBarStart;
   red->delta = nullptr;   // published again by this solve's first residual pass
 }
 

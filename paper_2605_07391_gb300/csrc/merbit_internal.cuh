@@ -23,6 +23,10 @@ constexpr int kMaxTpw = kMaxW / kWarps;             // tiles a warp reduces per 
 constexpr int kRedSlots = 64;       // spread slots of the grid-wide FP64 reductions
 constexpr uint32_t kMsb = 0x80000000u;
 constexpr uint32_t kSpinLimit = 1u << 22;           // bounded mbarrier waits
+// First value of a grid barrier's arrival count.  The count wraps (a solve of 2^31 updates passes
+// 2^32 arrivals many times), so counts are compared by their difference; starting just below the
+// wrap, every solve of a few updates passes it.
+constexpr uint32_t kBarStart = 0u - 1000u;
 constexpr int kMaxParts = 4096;                     // cap on persistent CTAs (partials array)
 
 // Per-plan device state for grid-wide reductions and kernel-side errors.
@@ -34,7 +38,7 @@ struct RedState {
   int iters;      // number of launches counted when `done` was set
   int inner_done; // refinement: the inner sweeps of the current step have converged
   int launches;   // SpMV launches that did work since the solve started
-  unsigned int bar;   // arrivals at the grid barriers of a cooperative solve
+  unsigned int bar;   // arrivals at the grid barriers of a cooperative solve, from kBarStart on
   const float* delta;   // refinement: buffer holding the latest inner iterate
 };
 
@@ -240,7 +244,7 @@ cudaError_t ppr_update(merbit_plan_s* p, const float* vals, const float* X, floa
                        cudaStream_t st);
 // All updates of a plain PageRank in one cooperative launch, from x0 (iterate k is in x0 for even k,
 // else in x1); *taken = false and nothing launched if the matrix does not fit the SMs' shared
-// memory.  hist[1] holds the first iterate's dangling mass, red->bar is zero; shares: 2 tile_num
+// memory.  hist[1] holds the first iterate's dangling mass, red->bar is kBarStart; shares: 2 tile_num
 // doubles of work space.
 cudaError_t pagerank_resident(merbit_plan_s* p, merbit_dtype dt, const void* vals, double alpha, double tol,
                               int max_iter, void* x0, void* x1, double* hist, double* shares, bool* taken,

@@ -171,9 +171,9 @@ __global__ void __launch_bounds__(kResWarps * 32, 1)
     atomicAdd(&g.red->bar, 1u);
   };
   auto wait = [&]() {                  // one thread; false if the barrier does not fill up
-    const unsigned int want = phase * (unsigned int)G;
+    const unsigned int want = kBarStart + phase * (unsigned int)G;
     for (uint32_t i = 0; i < kSpinLimit; ++i) {
-      if (*reinterpret_cast<volatile unsigned int*>(&g.red->bar) >= want) {
+      if ((int)(*reinterpret_cast<volatile unsigned int*>(&g.red->bar) - want) >= 0) {   // also past the wrap
         __threadfence();
         return true;
       }
