@@ -1,0 +1,48 @@
+"""Rows of a few tiles: an f32 product's error is that of sums within a tile and one rounding.
+
+Products of width 4 to 32 walk a tile in different orders, and a warp takes up to four tiles; the
+error must not grow with either.  The yardstick is a float32 model of the narrowest order: 14
+products a lane in turn, the 32 lanes of a tile pairwise, the tiles in 64 bits, one rounding.  A
+wider order has a few roundings more a tile: its root mean square may be 1.3 times the model's."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2605_07391_gb300 as mb
+
+pytestmark = pytest.mark.gpu
+ROWS, LEN, COLS = 6000, 1700, 200_000        # 22,800 tiles: units of four tiles
+
+
+def _model(prod):
+    """Row sums of float32 products (rows x LEN) in the order described above."""
+    rows = prod.shape[0]
+    pad = np.zeros((rows, -(-LEN // 448) * 448), np.float32)
+    pad[:, :LEN] = prod
+    lanes = np.zeros((rows, pad.shape[1] // 14), np.float32)
+    for k in range(14):
+        lanes += pad.reshape(rows, -1, 14)[:, :, k]
+    t = lanes.reshape(rows, -1, 32)
+    while t.shape[2] > 1:
+        t = t[:, :, ::2] + t[:, :, 1::2]
+    return t[:, :, 0].astype(np.float64).sum(1).astype(np.float32)
+
+
+def _rms(y, y64):
+    return float((((y.double() - y64) / y64) ** 2).mean().sqrt())
+
+
+@pytest.mark.parametrize("k", [4, 8, 13, 16, 32])
+def test_error_of_long_rows(cuda_device, k):
+    rng = np.random.default_rng(7)
+    row_ptr = torch.arange(0, ROWS * LEN + 1, LEN, dtype=torch.int32, device="cuda")
+    col = torch.from_numpy(rng.integers(0, COLS, ROWS * LEN).astype(np.int32)).cuda()
+    vals = torch.from_numpy(rng.random(ROWS * LEN).astype(np.float32)).cuda()
+    X = torch.from_numpy(rng.random((COLS, k)).astype(np.float32)).cuda()
+    p = mb.plan(row_ptr, col, ROWS, COLS)
+    y = mb.spmm(p, vals, X)
+    y64 = torch.stack([(vals.double() * X[:, c].double()[col.long()]).view(ROWS, LEN).sum(1) for c in range(k)], 1)
+    v, x, c0 = vals.cpu().numpy(), X[:, 0].cpu().numpy(), col.cpu().numpy()
+    prod = (v * x[c0]).reshape(ROWS, LEN)
+    model = _rms(torch.from_numpy(_model(prod)), torch.from_numpy(prod.astype(np.float64).sum(1)))
+    assert _rms(y, y64) <= 1.3 * model
