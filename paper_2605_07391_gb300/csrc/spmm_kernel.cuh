@@ -37,16 +37,6 @@
 
 namespace merbit {
 
-// s + x, and what the sum lost to rounding added to `lost` (Knuth's two-sum; nothing is lost by a
-// sum that is not finite).
-__device__ __forceinline__ void add_lost(float& s, float& lost, float x) {
-  const float t = s + x;
-  const float z = t - s;
-  const float e = (s - (t - z)) + (x - z);
-  lost += isfinite(t) ? e : 0.f;
-  s = t;
-}
-
 template <int VW> struct SpmmVec;
 template <> struct SpmmVec<1> {
   using T = float;

@@ -11,7 +11,8 @@
 //      are stored at once; the lane's first row end is kept (`head`);
 //   4. the runs open at the lanes' ends are joined by a segmented shuffle scan, a lane's
 //      first row totals its head plus the run that reaches it, and the run open after the
-//      tile is carried in a register into the next tile of the unit;
+//      tile is carried in a register into the next tile of the unit (with 4-byte sums, a
+//      second one holds what whole tiles of one row lost to rounding);
 //   5. the tile's rows go through the epilogue, consecutive lanes to consecutive rows, and
 //      the next tile's values are copied in.
 // So columns and values need one buffer each per warp: a column buffer is free once the
@@ -97,10 +98,20 @@ __device__ __forceinline__ void walk_issue(const T* src, void* dst, int xs, int 
   if (bytes) bulk_g2s(dst, src + sp.a0, bytes, bar, pol);
 }
 
+// s + x, and what the sum lost to rounding added to `lost` (Knuth's two-sum; nothing is lost by a
+// sum that is not finite).
+__device__ __forceinline__ void add_lost(float& s, float& lost, float x) {
+  const float t = s + x;
+  const float z = t - s;
+  const float e = (s - (t - z)) + (x - z);
+  lost += isfinite(t) ? e : 0.f;
+  s = t;
+}
+
 // The walk of one tile by a warp: a lane's steps (rm: right steps, dm: down steps; vp its first
 // value; xv its gathered x), the row sums into sy (y0: the row of the lane's first down step), the
-// runs joined across the lanes.  carry is the run that reaches the tile; the run open after it is
-// returned, in every lane.
+// runs joined across the lanes.  carry is the run that reaches the tile, added last where it ends;
+// the run open after the tile is returned, in every lane.
 template <typename VT, typename XT, typename AT>
 __device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax], uint32_t rm, uint32_t dm, AT* sy,
                                          int y0, AT carry, int lane) {
@@ -127,7 +138,6 @@ __device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax]
   // inclusive scan of the open runs; a lane that ends a row starts a new run
   const bool hd = dm != 0u;
   const uint32_t heads = __ballot_sync(0xffffffffu, hd);
-  if (lane == 0 && !hd) sum += carry;
   const uint32_t upto = heads & (0xffffffffu >> (31 - lane));
   const int dist = upto ? lane - (31 - __clz(upto)) : lane;   // lanes back to the run's start
   uint32_t run = ~heads & ~1u;                        // lanes that continue a run
@@ -140,7 +150,11 @@ __device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax]
   }
   // the run that reaches this lane's first row
   const AT up = __shfl_up_sync(0xffffffffu, sum, 1);
-  if (hd) sy[y0] = head + (lane == 0 ? carry : up);
+  if (hd) {
+    AT s = lane > 0 ? head + up : head;
+    if ((upto & (upto - 1u)) == 0u) s += carry;       // the tile's first row
+    sy[y0] = s;
+  }
   return __shfl_sync(0xffffffffu, sum, 31);
 }
 
@@ -320,6 +334,7 @@ __global__ void __launch_bounds__(kWalkThreads, CTAS)
   }
   uint32_t par = 0;
   AT carry = AT(0);                 // run open after the unit's tiles so far
+  float lost = 0.f;                 // what its sum lost to rounding (4-byte sums)
   int y_unit = (int)(tys & ~kMsb);  // the unit's first row
   bool ok = true;
   while (t >= 0) {
@@ -405,8 +420,15 @@ __global__ void __launch_bounds__(kWalkThreads, CTAS)
       }
     }
     AT* const sy = sy_end - n_t;                     // the tile's row sums
-    if (!single) carry = walk_lanes<VT, XT, AT>(sv + (vpad + xo), xv, rm, dm, sy, y0, carry, lane);
-    else carry += walk_row<VT, XT, AT>(sv + (vpad + lane), xv, xe - xs - lane);
+    if (!single) {
+      if constexpr (sizeof(AT) == 4) carry += lost;
+      carry = walk_lanes<VT, XT, AT>(sv + (vpad + xo), xv, rm, dm, sy, y0, carry, lane);
+      lost = 0.f;
+    } else {
+      const AT s = walk_row<VT, XT, AT>(sv + (vpad + lane), xv, xe - xs - lane);
+      if constexpr (sizeof(AT) == 4) add_lost(carry, lost, s);
+      else carry += s;
+    }
     __syncwarp();
 
     // ---- commit: the tile's rows; the unit's first row may have begun in another unit
@@ -416,9 +438,13 @@ __global__ void __launch_bounds__(kWalkThreads, CTAS)
       else epi.row(y_ws + r, s, p0, p1);
     }
     if (next_unit) {
-      if (lane == 0 && (int)tye < g.n_rows)
-        atomicAdd(g.tile_acc + __ldg(g.tile_slot + t + 1), static_cast<double>(carry));
+      if (lane == 0 && (int)tye < g.n_rows) {
+        double run = static_cast<double>(carry);
+        if constexpr (sizeof(AT) == 4) run += static_cast<double>(lost);
+        atomicAdd(g.tile_acc + __ldg(g.tile_slot + t + 1), run);
+      }
       carry = AT(0);
+      lost = 0.f;
       ++rd;
     }
     if constexpr (kVals) {
