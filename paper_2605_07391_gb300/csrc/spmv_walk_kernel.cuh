@@ -110,8 +110,8 @@ __device__ __forceinline__ void add_lost(float& s, float& lost, float x) {
 
 // The walk of one tile by a warp: a lane's steps (rm: right steps, dm: down steps; vp its first
 // value; xv its gathered x), the row sums into sy (y0: the row of the lane's first down step), the
-// runs joined across the lanes.  carry is the run that reaches the tile, added last where it ends;
-// the run open after the tile is returned, in every lane.
+// runs joined across the lanes.  carry is the run that reaches the tile (4-byte sums: added last
+// where it ends); the run open after the tile is returned, in every lane.
 template <typename VT, typename XT, typename AT>
 __device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax], uint32_t rm, uint32_t dm, AT* sy,
                                          int y0, AT carry, int lane) {
@@ -138,6 +138,9 @@ __device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax]
   // inclusive scan of the open runs; a lane that ends a row starts a new run
   const bool hd = dm != 0u;
   const uint32_t heads = __ballot_sync(0xffffffffu, hd);
+  if constexpr (sizeof(AT) == 8) {                    // one add fewer for the FP64 pipe
+    if (lane == 0 && !hd) sum += carry;
+  }
   const uint32_t upto = heads & (0xffffffffu >> (31 - lane));
   const int dist = upto ? lane - (31 - __clz(upto)) : lane;   // lanes back to the run's start
   uint32_t run = ~heads & ~1u;                        // lanes that continue a run
@@ -150,7 +153,9 @@ __device__ __forceinline__ AT walk_lanes(const VT* vp, const XT (&xv)[kSigmaMax]
   }
   // the run that reaches this lane's first row
   const AT up = __shfl_up_sync(0xffffffffu, sum, 1);
-  if (hd) {
+  if constexpr (sizeof(AT) == 8) {
+    if (hd) sy[y0] = head + (lane == 0 ? carry : up);
+  } else if (hd) {
     AT s = lane > 0 ? head + up : head;
     if ((upto & (upto - 1u)) == 0u) s += carry;       // the tile's first row
     sy[y0] = s;
