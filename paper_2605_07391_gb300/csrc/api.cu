@@ -199,7 +199,7 @@ merbit_status convert_typed(const S* src, void* dst, merbit_dtype ddt, int64_t n
   int k = 0;
   if (auto_scale && ddt == MERBIT_F16 && nnz > 0) {
     unsigned long long* d = nullptr;
-    MB_TRY(cudaMalloc(&d, sizeof(unsigned long long)));
+    MB_TRY(dev_malloc(reinterpret_cast<void**>(&d), sizeof(unsigned long long)));
     unsigned long long bits = 0;
     cudaError_t e = cudaMemsetAsync(d, 0, sizeof(bits), st);
     if (e == cudaSuccess) {

@@ -41,8 +41,8 @@ merbit_status merbit_autotune_sigma(const int32_t* row_ptr, const int32_t* col_i
   const size_t es = dtype == MERBIT_F64 ? 8 : 4;
   void *x = nullptr, *y = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaError_t e = cudaMalloc(&x, es * (size_t)std::max<int64_t>(n_cols, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&y, es * (size_t)std::max<int64_t>(n_rows, 1));
+  cudaError_t e = dev_malloc(&x, es * (size_t)std::max<int64_t>(n_cols, 1));
+  if (e == cudaSuccess) e = dev_malloc(&y, es * (size_t)std::max<int64_t>(n_rows, 1));
   if (e == cudaSuccess) e = cudaMemsetAsync(x, 0, es * (size_t)std::max<int64_t>(n_cols, 1), st);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -110,8 +110,8 @@ merbit_status merbit_autotune(const int32_t* row_ptr, const int32_t* col_idx, in
   const size_t es = xdt == MERBIT_F64 ? 8 : 4;
   void *x = nullptr, *y = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaError_t e = cudaMalloc(&x, es * (size_t)std::max<int64_t>(n_cols, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&y, es * (size_t)std::max<int64_t>(n_rows, 1));
+  cudaError_t e = dev_malloc(&x, es * (size_t)std::max<int64_t>(n_cols, 1));
+  if (e == cudaSuccess) e = dev_malloc(&y, es * (size_t)std::max<int64_t>(n_rows, 1));
   if (e == cudaSuccess) e = cudaMemsetAsync(x, 0, es * (size_t)std::max<int64_t>(n_cols, 1), st);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);

@@ -682,7 +682,7 @@ merbit_status merbit_batch_pagerank(merbit_batch_t b, merbit_dtype dtype, const 
       cudaFree(b->x1);
       b->x1 = nullptr;
       b->x1_bytes = 0;
-      e = cudaMalloc(&b->x1, es * (size_t)std::max<int64_t>(b->n, 1));
+      e = dev_malloc(&b->x1, es * (size_t)std::max<int64_t>(b->n, 1));
       if (e == cudaSuccess) b->x1_bytes = es * (size_t)b->n;
     }
     cudaStream_t cap = nullptr;

@@ -82,8 +82,8 @@ cudaError_t get_state(const merbit_plan_s* p, size_t xb, size_t yb, AsyncState**
       cudaFree(a->x[s]);
       cudaFree(a->y[s]);
       a->x[s] = a->y[s] = nullptr;
-      e = cudaMalloc(&a->x[s], xb);
-      if (e == cudaSuccess) e = cudaMalloc(&a->y[s], yb);
+      e = dev_malloc(&a->x[s], xb);
+      if (e == cudaSuccess) e = dev_malloc(&a->y[s], yb);
     }
     if (e == cudaSuccess) {
       a->xb = xb;

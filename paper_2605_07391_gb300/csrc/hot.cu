@@ -121,11 +121,11 @@ merbit_status build_hot_table(merbit_plan_s* p, int max_hot, double min_cover, c
     cudaFree(sel_cnt);
     cudaFree(nsel);
   };
-  cudaError_t e = cudaMalloc(&cnt, sizeof(uint32_t) * (size_t)n);
-  if (e == cudaSuccess) e = cudaMalloc(&hist, sizeof(uint32_t) * kHistBins);
-  if (e == cudaSuccess) e = cudaMalloc(&sel_col, sizeof(int32_t) * (size_t)max_hot);
-  if (e == cudaSuccess) e = cudaMalloc(&sel_cnt, sizeof(uint32_t) * (size_t)max_hot);
-  if (e == cudaSuccess) e = cudaMalloc(&nsel, sizeof(int));
+  cudaError_t e = dev_malloc(reinterpret_cast<void**>(&cnt), sizeof(uint32_t) * (size_t)n);
+  if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&hist), sizeof(uint32_t) * kHistBins);
+  if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&sel_col), sizeof(int32_t) * (size_t)max_hot);
+  if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&sel_cnt), sizeof(uint32_t) * (size_t)max_hot);
+  if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&nsel), sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (size_t)n, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kHistBins, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(nsel, 0, sizeof(int), st);
@@ -190,8 +190,8 @@ merbit_status build_hot_table(merbit_plan_s* p, int max_hot, double min_cover, c
     cleanup();
     return MERBIT_OK;
   }
-  e = cudaMalloc(&p->hot_list, sizeof(int32_t) * (size_t)ns);
-  if (e == cudaSuccess) e = cudaMalloc(&p->col_hot, sizeof(int32_t) * (size_t)nnz);
+  e = dev_malloc(reinterpret_cast<void**>(&p->hot_list), sizeof(int32_t) * (size_t)ns);
+  if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&p->col_hot), sizeof(int32_t) * (size_t)nnz);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(p->hot_list, list.data(), sizeof(int32_t) * (size_t)ns, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {

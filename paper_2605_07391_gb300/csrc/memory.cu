@@ -4,7 +4,8 @@
 // new pattern (two plans and a transpose, 26 device allocations at R-MAT scale 20) spent 1.1 of
 // its 1.88 ms in them; from the pool a block costs 1 us, and the set-up 0.76 ms.  The pool keeps at
 // most kPoolKeep bytes that no object uses: what is above that goes back to the driver at the next
-// synchronisation, all of it when an allocation fails, and the rest when the process ends.
+// synchronisation, all of it when an allocation of the library fails, and the rest when the process
+// ends.
 #include <mutex>
 #include <unordered_map>
 
@@ -65,6 +66,18 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
     cudaMemPoolTrimTo(pool, 0);
   }
   return cudaMalloc(p, bytes ? bytes : 1);
+}
+
+cudaError_t dev_malloc(void** p, size_t bytes) {
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const cudaMemPool_t pool = pool_of(dev);
+  if (!pool) return e;
+  cudaGetLastError();
+  cudaMemPoolTrimTo(pool, 0);
+  return cudaMalloc(p, bytes);
 }
 
 cudaError_t device_wait(int device) {

@@ -190,6 +190,9 @@ struct SweepParams {
 // after the work that uses it has been waited for.
 cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st);
 
+// cudaMalloc, tried again without the pool's idle memory when there is none left.
+cudaError_t dev_malloc(void** p, size_t bytes);
+
 // While one lives, unsafe calls (cudaMalloc, cudaFree) of this thread leave the captures of any thread alone.
 struct RelaxedCalls {
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;

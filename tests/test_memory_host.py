@@ -61,3 +61,28 @@ def test_state_is_clear_after_a_give_up(lib, kind):
     assert st == 6, lib.merbit_last_error()
     assert not state.any()
     getattr(lib, "merbit_batch_destroy" if kind == "batch" else "merbit_plan_destroy")(h)
+
+
+@pytest.mark.parametrize("call", ["autotune", "hot", "host_async"])
+def test_idle_pool_memory_is_given_back(lib, call):
+    """What the pool holds for later does not make another allocation of the library fail."""
+    lib.fake_reset()
+    m = fr.Pattern(lib)
+    h = m.plan()
+    for p in [m.plan() for _ in range(12)]:
+        lib.merbit_plan_destroy(p)
+    assert lib.fake_idle() > 500_000
+    lib.fake_limit(100)
+    v, x, y = np.zeros(m.nnz), np.zeros(m.n), np.zeros(m.n)
+    vp, i64 = ctypes.c_void_p, ctypes.c_int64
+    if call == "autotune":
+        cand, best = (ctypes.c_int * 1)(14), ctypes.c_int()
+        st = lib.merbit_autotune_sigma(*m.args(), 0, vp(v.ctypes.data + -v.ctypes.data % 16), cand, 1, 1, None,
+                                       ctypes.byref(best), None)
+    elif call == "hot":
+        st = lib.merbit_plan_set_hot_columns(h, 64, ctypes.c_double(0.0), None, None, None)
+    else:
+        st = lib.merbit_spmv_host_async(h, 0, vp(v.ctypes.data + -v.ctypes.data % 16), vp(x.ctypes.data), vp(y.ctypes.data),
+                                        None)
+    assert st == 0, (st, lib.merbit_last_error())
+    lib.merbit_plan_destroy(h)
