@@ -264,7 +264,9 @@ size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 merbit_status ensure_spmm_acc(merbit_plan_s* p, cudaStream_t st) {
   if (p->spmm_acc) return MERBIT_OK;
   const size_t bytes = sizeof(double) * 32 * (size_t)spmm_acc_sets(p);
-  MB_TRY(cudaMalloc(&p->spmm_acc, bytes));
+  void* acc = nullptr;
+  MB_TRY(dev_alloc(&acc, bytes, st));
+  p->spmm_acc = static_cast<double*>(acc);
   MB_TRY(cudaMemsetAsync(p->spmm_acc, 0, bytes, st));
   return MERBIT_OK;
 }
@@ -517,12 +519,12 @@ merbit_status merbit_spmm(merbit_plan_t p, const float* vals, const float* X, fl
   if (!aligned(X, 4) || !aligned(Y, 4)) return fail(MERBIT_EINVAL, "X / Y must be 4-byte aligned");
   if ((int64_t)p->n_cols * ldx >= ((int64_t)1 << 40)) return fail(MERBIT_EINVAL, "X too large");
   cudaStream_t st = as_stream(stream);
-  if (merbit_status s = ensure_spmm_acc(p, st)) return s;
   // one contiguous column is the plain product (R-MAT scale 21: 0.113 ms, one-column slices 0.228)
   if (k == 1 && ldx == 1 && ldy == 1) {
     MB_TRY(spmv_plain_f32(p, vals, X, Y, st));
     return MERBIT_OK;
   }
+  if (merbit_status s = ensure_spmm_acc(p, st)) return s;
   MB_TRY(spmm_plain_f32(p, vals, X, k, ldx, Y, ldy, p->spmm_acc, st));
   return MERBIT_OK;
 }

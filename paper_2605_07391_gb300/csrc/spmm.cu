@@ -47,10 +47,10 @@ float* pack_buffer(merbit_plan_s* p, int kc, cudaStream_t st) {
   }
   const size_t need = sizeof(float) * (size_t)kc * (size_t)p->n_cols;
   if (p->spmm_pack_bytes < need) {
-    cudaFree(p->spmm_pack);
+    if (p->spmm_pack) dev_free(p->device, {p->spmm_pack});
     p->spmm_pack = nullptr;
     p->spmm_pack_bytes = 0;
-    if (cudaMalloc(&p->spmm_pack, need) != cudaSuccess) {
+    if (dev_alloc(&p->spmm_pack, need, st) != cudaSuccess) {
       cudaGetLastError();
       p->spmm_pack = nullptr;
       return nullptr;

@@ -86,3 +86,18 @@ def test_idle_pool_memory_is_given_back(lib, call):
                                         None)
     assert st == 0, (st, lib.merbit_last_error())
     lib.merbit_plan_destroy(h)
+
+
+@pytest.mark.parametrize("k", [1, 8, 13])
+def test_first_spmm_of_a_plan_takes_pool_memory(lib, k):
+    lib.fake_reset()
+    m = fr.Pattern(lib)
+    h = m.plan()
+    v, X, Y = np.zeros(m.nnz + 4, np.float32), np.zeros(m.n * k + 4, np.float32), np.zeros(m.n * k + 4, np.float32)
+    at = [ctypes.c_void_p(t.ctypes.data + -t.ctypes.data % 16) for t in (v, X, Y)]
+    before, used = lib.fake_mallocs(), lib.fake_used()
+    k64 = ctypes.c_int64(k)
+    assert lib.merbit_spmm(h, *at, k64, k64, k64, None) == 0, lib.merbit_last_error()
+    assert lib.fake_mallocs() == before
+    assert (lib.fake_used() == used) == (k == 1)      # one column needs no accumulators
+    lib.merbit_plan_destroy(h)
