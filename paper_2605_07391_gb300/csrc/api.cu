@@ -62,7 +62,7 @@ void free_plan(merbit_plan_s* p) {
   host_async_release(p);
   free_hot_table(p);
   dev_free(p->device, {p->block, p->dangling_bits, p->scratch, p->hist, p->x_stage, p->y_stage, p->spmm_acc,
-                       p->spmm_pack});
+                       p->spmm_pack[0], p->spmm_pack[1], p->spmm_pack[2], p->spmm_pack[3]});
   if (p->host_pinned) cudaFreeHost(p->host_pinned);
   delete p;
 }

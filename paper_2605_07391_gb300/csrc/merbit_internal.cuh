@@ -114,8 +114,10 @@ struct merbit_plan_s {
   size_t x_stage_bytes = 0, y_stage_bytes = 0;
   void* host_pinned = nullptr;           // small pinned block for state read-back (on first use)
   double* spmm_acc = nullptr;            // spmm_acc_sets x 32 FP64 boundary accumulators of the SpMM
-  void* spmm_pack = nullptr;             // padded copy of up to 32 columns of an unaligned X
-  size_t spmm_pack_bytes = 0;
+  // padded copies of 4, 8, 16 and 32 columns of an unaligned X; bit w of spmm_pack_recorded: a
+  // captured launch uses copy w, which stays until the plan goes
+  void* spmm_pack[4] = {nullptr, nullptr, nullptr, nullptr};
+  uint32_t spmm_pack_recorded = 0u;
 
   merbit::Geometry geom() const {
     merbit::Geometry g;
