@@ -36,6 +36,10 @@ constexpr int kSortItems = 12;                       // nonzeros per thread
 constexpr int kTile = kSortThreads * kSortItems;     // nonzeros per CTA
 constexpr int kDigitBits = 11;                       // largest digit
 constexpr int kScanThreads = 256;
+// Rows that start inside a tile are walked by its CTA, 512 at a time, up to this many; beyond that
+// (runs of empty rows) each nonzero searches its row: 15 ms for 2^24 empty rows in one tile, walked;
+// the search takes some 25 steps.
+constexpr int kRowsWalked = 2 * kTile;
 
 // Exclusive scan of one value per thread over the CTA (whole warps); *total gets the sum.
 __device__ __forceinline__ uint32_t cta_exclusive_scan(uint32_t v, uint32_t* warp_tot, uint32_t* total) {
@@ -170,40 +174,54 @@ __global__ void __launch_bounds__(kSortThreads, 2)
   for (int i = tid; i < kSortWarps * bins / 2; i += kSortThreads) wz[i] = 0u;
   uint32_t row[FIRST ? kSortItems : 1];
   if constexpr (FIRST) {
-    // rows of the tile's nonzeros: every row that starts inside the tile marks its first nonzero
-    // (the last of several rows that start there wins: the others are empty), then a running maximum
     const int r0 = __ldg(tile_row + blockIdx.x);
-    for (int i = tid; i < kTile; i += kSortThreads) stage[i] = 0u;
-    __syncthreads();
-    for (int64_t r = (int64_t)r0 + 1 + tid; r < n_rows; r += kSortThreads) {
-      const int64_t p = (int64_t)__ldg(row_ptr + r) - t0;
-      if (p >= count) break;
-      atomicMax(&stage[p], (uint32_t)(r - r0));
-    }
-    __syncthreads();
-    // a warp takes its own 512 nonzeros, 32 at a time, after the maxima of the warps before
-    uint32_t m = 0;
+    const int r1 = (int)blockIdx.x + 1 < num_tiles ? __ldg(tile_row + blockIdx.x + 1) : (int)n_rows - 1;
+    if (r1 - r0 > kRowsWalked) {
+      // a long run of empty rows: a search for every nonzero, a step of all of a thread's at a time
 #pragma unroll
-    for (int it = 0; it < kSortItems; ++it) {
-      row[it] = stage[w0 + it * 32];
-      m = max(m, row[it]);
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) warp_tot[warp] = m;
-    __syncthreads();
-    uint32_t run = 0;
-    for (int w = 0; w < warp; ++w) run = max(run, warp_tot[w]);
+      for (int it = 0; it < kSortItems; ++it) row[it] = (uint32_t)r0;
+      for (uint32_t s = 1u << (31 - __clz(r1 - r0)); s > 0u; s >>= 1) {
 #pragma unroll
-    for (int it = 0; it < kSortItems; ++it) {
-      uint32_t inc = row[it];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc = max(inc, y);
+        for (int it = 0; it < kSortItems; ++it) {
+          const uint32_t r = row[it] + s;              // rows stay below 2^31, steps below 2^31
+          if (r <= (uint32_t)r1 && (int64_t)__ldg(row_ptr + r) <= t0 + w0 + it * 32) row[it] = r;
+        }
       }
-      inc = max(inc, run);
-      run = __shfl_sync(0xffffffffu, inc, 31);
-      row[it] = inc + (uint32_t)r0;
+    } else {
+      // rows of the tile's nonzeros: every row that starts inside the tile marks its first nonzero
+      // (the last of several rows that start there wins: the others are empty), then a running maximum
+      for (int i = tid; i < kTile; i += kSortThreads) stage[i] = 0u;
+      __syncthreads();
+      for (int64_t r = (int64_t)r0 + 1 + tid; r < n_rows; r += kSortThreads) {
+        const int64_t p = (int64_t)__ldg(row_ptr + r) - t0;
+        if (p >= count) break;
+        atomicMax(&stage[p], (uint32_t)(r - r0));
+      }
+      __syncthreads();
+      // a warp takes its own 384 nonzeros, 32 at a time, after the maxima of the warps before
+      uint32_t m = 0;
+#pragma unroll
+      for (int it = 0; it < kSortItems; ++it) {
+        row[it] = stage[w0 + it * 32];
+        m = max(m, row[it]);
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) warp_tot[warp] = m;
+      __syncthreads();
+      uint32_t run = 0;
+      for (int w = 0; w < warp; ++w) run = max(run, warp_tot[w]);
+#pragma unroll
+      for (int it = 0; it < kSortItems; ++it) {
+        uint32_t inc = row[it];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc = max(inc, y);
+        }
+        inc = max(inc, run);
+        run = __shfl_sync(0xffffffffu, inc, 31);
+        row[it] = inc + (uint32_t)r0;
+      }
     }
   }
   __syncthreads();
