@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(256)
 
 constexpr int kRowsPerWarp = 1024;
 constexpr int kRowsInFlight = 8;      // per lane
+constexpr int kSmallGraphs = 32;      // a warp's rows in more graphs than this: a row a lane
 
 // acc[2g] += sum |y - x|, acc[2g + 1] += sum of y over dangling rows, for active graphs.
 // A warp takes kRowsPerWarp consecutive rows, graph by graph: eight rows a lane in flight, and one
@@ -240,7 +241,46 @@ __global__ void __launch_bounds__(256)
        c += warps) {
     const int64_t r_end = (c + 1) * kRowsPerWarp < n ? (c + 1) * kRowsPerWarp : n;
     int64_t r0 = c * kRowsPerWarp;
-    for (int g = graph_of(off, G, (int)r0); r0 < r_end; ++g) {
+    int g = graph_of(off, G, (int)r0);
+    if (__ldg(off + min(g + kSmallGraphs, G)) < r_end) {
+      // small graphs: a row a lane, the lanes of a graph joined by a segmented scan
+      for (; r0 < r_end; r0 += 32) {
+        const int64_t r = r0 + lane;
+        const bool in = r < r_end;
+        int lo = g, hi = min(g + 32, G);                 // 32 rows lie in 32 graphs at most
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (in && (int64_t)__ldg(off + mid) <= r) lo = mid; else hi = mid;
+        }
+        double p0 = 0.0, p1 = 0.0;
+        const bool live = in && conv[lo] < 0;
+        if (live) {
+          const T yr = y[r];
+          p0 = fabs(static_cast<double>(yr) - static_cast<double>(x[r]));
+          if (is_dangling(dang, (int)r)) p1 = static_cast<double>(yr);
+        }
+        const int key = in ? lo : G;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double u0 = __shfl_up_sync(0xffffffffu, p0, o), u1 = __shfl_up_sync(0xffffffffu, p1, o);
+          const int k = __shfl_up_sync(0xffffffffu, key, o);
+          if (lane >= o && k == key) {
+            p0 += u0;
+            p1 += u1;
+          }
+        }
+        const int next = __shfl_down_sync(0xffffffffu, key, 1);
+        if (live && (lane == 31 || next != key)) {
+          if (p0 != 0.0) atomicAdd(acc + 2 * lo, p0);
+          if (p1 != 0.0) atomicAdd(acc + 2 * lo + 1, p1);
+        }
+        // the graph of the next row: this window's last one, or the one after it
+        g = __shfl_sync(0xffffffffu, lo, 31);
+        if (r0 + 32 < r_end && (int64_t)__ldg(off + g + 1) <= r0 + 32) ++g;
+      }
+      continue;
+    }
+    for (; r0 < r_end; ++g) {
       const int64_t hi = __ldg(off + g + 1);
       const int64_t e = hi < r_end ? hi : r_end;
       if (conv[g] < 0) {
