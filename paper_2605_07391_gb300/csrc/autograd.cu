@@ -126,6 +126,54 @@ __global__ void __launch_bounds__(kSddmmWarps * 32, sizeof(T) == 8 ? 3 : 4)
   }
 }
 
+// The same with a thread per lane of the schedule, for sigma below kSddmmTileSigma: a tile is then too
+// little for a warp (sigma 1: 32 steps), and a lane's nonzeros hardly spread.  R-MAT scale 20, this
+// and a warp per tile: f32, sigma 1 105 us (227), 2 70 (107), 3 69 (80), 4 76 (69); f64, sigma 1 115
+// (237), 2 87 (123), 3 94 (92).
+template <typename T>
+constexpr int kSddmmTileSigma = sizeof(T) == 8 ? 3 : 4;
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+    sddmm_lanes_kernel(const Geometry g, const T* __restrict__ gv, const T* __restrict__ x, T scale,
+                       T* __restrict__ out) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < g.lane_num; j += stride) {
+    const int ti = (int)(j / kOmega);
+    const LaneDesc d = decode_lane(g, load_desc(g, j));
+    int xk = (int)__ldg(g.tile_x + ti) + d.xo;
+    int row = (int)(__ldg(g.tile_y + ti) & ~kMsb) + d.yo;
+    const int64_t left = (int64_t)g.steps - j * g.sigma;
+    const int len = left < g.sigma ? (int)left : g.sigma;
+    T gr = row < g.n_rows ? scale * gv[row] : T(0);
+    for (int k = 0; k < len; ++k) {
+      if ((d.flags >> k) & 1u) {
+        ++row;
+        gr = row < g.n_rows ? scale * gv[row] : T(0);
+      } else {
+        out[xk] = gr * x[__ldg(g.col + xk)];
+        ++xk;
+      }
+    }
+  }
+}
+
+template <typename T>
+cudaError_t sddmm_typed(const merbit_plan_s* p, const T* g, const T* x, T scale, T* out, cudaStream_t st) {
+  if (p->sigma < kSddmmTileSigma<T>) {
+    const int grid = (int)std::min<int64_t>((p->lane_num + 255) / 256, (int64_t)p->num_sms * 16);
+    sddmm_lanes_kernel<T><<<grid, 256, 0, st>>>(p->geom(), g, x, scale, out);
+    return cudaGetLastError();
+  }
+  const size_t smem = kSddmmWarps * ((size_t)kOmega * p->sigma + 2) * sizeof(T);
+  const size_t most = kSddmmWarps * ((size_t)kOmega * kSigmaMax64 + 2) * sizeof(T);
+  int grid = persistent_grid(reinterpret_cast<const void*>(sddmm_kernel<T>), kSddmmWarps * 32, smem, most, p->num_sms);
+  if (grid <= 0) return cudaErrorInvalidConfiguration;
+  grid = (int)std::min<int64_t>(grid, (p->tile_num + kSddmmWarps - 1) / kSddmmWarps);
+  sddmm_kernel<T><<<grid, kSddmmWarps * 32, smem, st>>>(p->geom(), g, x, scale, out);
+  return cudaGetLastError();
+}
+
 template <typename T, bool ABS>
 __global__ void vec_sum_kernel(const T* __restrict__ x, int64_t n, double* out) {
   double s = 0.0;
@@ -157,22 +205,11 @@ cudaError_t spmv_adj_f64(const merbit_plan_s* p, const double* vals, const doubl
 cudaError_t sddmm(const merbit_plan_s* p, merbit_dtype dt, const void* g, const void* x,
                   double scale, void* out, cudaStream_t st) {
   if (p->lane_num == 0) return cudaSuccess;
-  const size_t smem = kSddmmWarps * ((size_t)kOmega * p->sigma + 2) * (dt == MERBIT_F64 ? 8 : 4);
-  const size_t most = kSddmmWarps * ((size_t)kOmega * kSigmaMax64 + 2) * (dt == MERBIT_F64 ? 8 : 4);
-  const void* kern = dt == MERBIT_F64 ? reinterpret_cast<const void*>(sddmm_kernel<double>)
-                                      : reinterpret_cast<const void*>(sddmm_kernel<float>);
-  int grid = persistent_grid(kern, kSddmmWarps * 32, smem, most, p->num_sms);
-  if (grid <= 0) return cudaErrorInvalidConfiguration;
-  grid = (int)std::min<int64_t>(grid, (p->tile_num + kSddmmWarps - 1) / kSddmmWarps);
   if (dt == MERBIT_F64)
-    sddmm_kernel<double><<<grid, kSddmmWarps * 32, smem, st>>>(p->geom(), static_cast<const double*>(g),
-                                                               static_cast<const double*>(x), scale,
-                                                               static_cast<double*>(out));
-  else
-    sddmm_kernel<float><<<grid, kSddmmWarps * 32, smem, st>>>(p->geom(), static_cast<const float*>(g),
-                                                              static_cast<const float*>(x),
-                                                              static_cast<float>(scale), static_cast<float*>(out));
-  return cudaGetLastError();
+    return sddmm_typed<double>(p, static_cast<const double*>(g), static_cast<const double*>(x), scale,
+                               static_cast<double*>(out), st);
+  return sddmm_typed<float>(p, static_cast<const float*>(g), static_cast<const float*>(x), static_cast<float>(scale),
+                            static_cast<float*>(out), st);
 }
 
 cudaError_t vec_sum(const void* x, merbit_dtype dt, int64_t n, double* out, bool absolute,
