@@ -530,8 +530,11 @@ inline int walk_unit(int64_t tiles, int64_t warps, int W) {
   return c;
 }
 
-// Products of at most this many unit boundaries are finished by the kernel's last CTA.
-constexpr int64_t kWalkFoldMax = 1024;
+// Products of at most this many unit boundaries are finished by the kernel's last CTA: a launch less,
+// but one CTA for all of them.  R-MAT-like graphs, refinement to 1e-10 with this limit at 1,024 and
+// at 2,048: 1,237 tiles 2.27 and 2.10 ms, 1,439 tiles 2.69 and 2.55, 1,718 and 1,897 tiles level;
+// BiCGSTAB, an iteration: 1,499 tiles 59.2 and 59.9 us.
+constexpr int64_t kWalkFoldMax = 1440;
 
 template <typename VT, typename XT, typename AT, typename Epi>
 cudaError_t launch_walk(const merbit_plan_s* p, const VT* vals, const XT* x, const Epi& epi, cudaStream_t st) {
