@@ -255,11 +255,15 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
     if (lane == 0)
       walk_issue(static_cast<const int32_t*>(src), dst, a, b, g.nnz, &bars[warp][which], policy_evict_first());
   };
-  auto add_acc = [&](int tile, const VT& v) {
+  auto add_acc = [&](int tile, const VT& v, const VT& lost) {
     double* a = acc + (size_t)spmm_set(g, tile) * KC + c;
 #pragma unroll
     for (int i = 0; i < VW; ++i)
-      if (i < left) atomicAdd(a + i, (double)V::get(v, i));
+      if (i < left) {
+        double q = (double)V::get(v, i);
+        if (V::get(lost, i) != 0.f) q += (double)V::get(lost, i);
+        atomicAdd(a + i, q);
+      }
   };
 
   int rd = 0;
@@ -413,7 +417,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
             V::add(in, V::load_shared(s_carry));
           }
           if (y0 == y_unit) {
-            if (c_ok) add_acc(t_start, in);
+            if (c_ok) add_acc(t_start, in, V::zero());
           } else {
             spmm_store_if<VW, YVEC, SCALED>(c_ok, y_row(y0), in, out.scale, left);
           }
@@ -433,14 +437,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
     if (next_unit) {
       const int y_end = (int)(__shfl_sync(0xffffffffu, meta, 3) & ~kMsb);
       if (gl == 0) {
-        if (c_ok && y_end < g.n_rows) {
-          add_acc(t + 1, V::load_shared(s_carry));
-          const VT lost = V::load_shared(s_lost);
-          bool any_lost = false;
-#pragma unroll
-          for (int i = 0; i < VW; ++i) any_lost |= V::get(lost, i) != 0.f;
-          if (any_lost) add_acc(t + 1, lost);
-        }
+        if (c_ok && y_end < g.n_rows) add_acc(t + 1, V::load_shared(s_carry), V::load_shared(s_lost));
         V::store_shared(s_carry, V::zero());
         V::store_shared(s_lost, V::zero());
       }
