@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
   using VT = typename V::T;
   constexpr int T = KC / VW;                   // threads per lane, one slice of VW columns each
   constexpr int L = 32 / T;                    // lanes walked at once (one pass)
-  constexpr int U1 = 8;                        // row slices per round of a single-row tile
+  constexpr int U1 = VW == 1 ? 16 : 8;         // row slices per round of a single-row tile
   __shared__ __align__(8) uint64_t bars[kSpmmWarps][2];
   extern __shared__ __align__(128) unsigned char dyn_smem[];
 
