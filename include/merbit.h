@@ -178,7 +178,8 @@ merbit_status merbit_plan_set_hot_columns(merbit_plan_t plan, int max_hot, doubl
  * included when that launch would use it.  The column stream is read coalesced; every
  * gathered value is summed and each CTA writes its sum to sink (device, at least 4096
  * entries of xdt).  Timing it beside the product gives the cost of the gathers at the
- * kernel's shared-memory footprint.  Asynchronous on `stream`.  Errors: EINVAL, ECUDA.
+ * split kernel's shared-memory footprint (the lane-walk kernel, the automatic choice of
+ * most plans, leaves L1 another share).  Asynchronous on `stream`.  Errors: EINVAL, ECUDA.
  */
 merbit_status merbit_gather_probe(merbit_plan_t plan, merbit_dtype xdt, const void* x, void* sink,
                                   void* stream);
@@ -227,13 +228,18 @@ merbit_status merbit_spmv_ex(merbit_plan_t plan, merbit_dtype vals_dtype, merbit
  * with ldy >= k, all f32 device pointers; vals f32, 16-byte aligned.  The plan
  * must have 8 tiles per block and sigma <= 14.  Columns are processed in chunks of
  * 32, 16, 8 or 4; each nonzero's column index and value are read once per chunk and
- * the gathered row slice X[col, chunk] serves the whole chunk.  When k, ldx and ldy
- * are multiples of 4 and X, Y are 16-byte aligned the slices are read as 16-byte
- * vectors (32-byte ones in chunks of 16 and 32 when k and ldx are also multiples of 8
- * and X is 32-byte aligned), otherwise element by element.  Y's first k columns are
- * fully overwritten (rows of A with no nonzeros get 0).
- * Asynchronous on `stream`; allocates (once per plan) a (block_num + 1) x 32
- * FP64 accumulator for rows shared between blocks.  A stage wait that gives up
+ * the gathered row slice X[col, chunk] serves the whole chunk.  When k and ldx are
+ * multiples of 4 and X is 16-byte aligned the slices are read as 16-byte vectors.
+ * Other X are copied into padded rows first, a chunk at a time, when the matrix has at
+ * least 3 nonzeros per column, and read element by element when it has fewer or there
+ * is no memory for the copy.  One contiguous column (k = ldx = ldy = 1) is merbit_spmv's
+ * product.  Y's first k columns are fully overwritten (rows of A with no nonzeros get 0).
+ * Asynchronous on `stream`.  The plan keeps, from their first use on, 32 FP64
+ * accumulators for every unit of one to four tiles (rows shared between units), and for
+ * unaligned X a copy of the widest chunk used (16, 32, 64 or 128 bytes per column of A;
+ * a copy that a captured launch uses stays beside a wider one).  Under stream capture
+ * the accumulators must exist (an earlier product on the plan with k > 1, or
+ * merbit_ppr).  A stage wait that gives up
  * (bounded; see merbit_plan_set_wait_limit) is reported by merbit_plan_sync as
  * MERBIT_EDEVICE.  Errors: EINVAL (NULL pointers, k < 0, ldx < k, ldy < k,
  * misaligned vals, a plan of other than 8 tiles per block or sigma > 14), ENOMEM,

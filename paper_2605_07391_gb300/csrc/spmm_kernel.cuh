@@ -26,8 +26,8 @@
 // warps, 14 slices of 16 bytes a thread: 114 KB an SM).  Multiply-adds and stores are predicated
 // on the descriptor's bits instead of branched over, and no table, arrival count or block barrier
 // joins the warps: 2.6 warp instructions per nonzero at k = 8 instead of 3.2.  R-MAT scale 21
-// (32.4 M nonzeros), before and after: k = 4 0.189 / 0.163 ms, k = 8 0.224 / 0.192, k = 16 0.302 /
-// 0.271, k = 32 0.495 / 0.466.
+// (32.4 M nonzeros), before and after: k = 4 0.189 / 0.170 ms, k = 8 0.224 / 0.192, k = 16 0.302 /
+// 0.275, k = 32 0.495 / 0.474.
 #pragma once
 
 #include <climits>
@@ -41,7 +41,6 @@ template <int VW> struct SpmmVec;
 template <> struct SpmmVec<1> {
   using T = float;
   static __device__ __forceinline__ T zero() { return 0.f; }
-  static __device__ __forceinline__ T load(const float* p) { return __ldg(p); }
   static __device__ __forceinline__ T load_plain(const float* p) { return *p; }
   static __device__ __forceinline__ void store(float* p, const float (&a)[1]) { *p = a[0]; }
   static __device__ __forceinline__ T load_shared(const float* p) { return *p; }
@@ -52,7 +51,6 @@ template <> struct SpmmVec<1> {
   }
   static __device__ __forceinline__ void fma(float w, const T& x, T& s) { s = fmaf(w, x, s); }
   static __device__ __forceinline__ float get(const T& v, int) { return v; }
-  static __device__ __forceinline__ T from(const float (&a)[1]) { return a[0]; }
   static __device__ __forceinline__ void add(T& s, const T& x) { s += x; }
   static __device__ __forceinline__ void add_exact(T& s, T& lost, const T& x) { add_lost(s, lost, x); }
   static __device__ __forceinline__ T shfl_up(const T& v, int d) {
@@ -61,16 +59,10 @@ template <> struct SpmmVec<1> {
   static __device__ __forceinline__ T shfl_xor(const T& v, int d) {
     return __shfl_xor_sync(0xffffffffu, v, d);
   }
-  static __device__ __forceinline__ T shfl(const T& v, int src) {
-    return __shfl_sync(0xffffffffu, v, src);
-  }
 };
 template <> struct SpmmVec<4> {
   using T = float4;
   static __device__ __forceinline__ T zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-  static __device__ __forceinline__ T load(const float* p) {
-    return __ldg(reinterpret_cast<const float4*>(p));
-  }
   static __device__ __forceinline__ T load_plain(const float* p) {
     return *reinterpret_cast<const float4*>(p);
   }
@@ -93,9 +85,6 @@ template <> struct SpmmVec<4> {
   static __device__ __forceinline__ float get(const T& v, int i) {
     return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
   }
-  static __device__ __forceinline__ T from(const float (&a)[4]) {
-    return make_float4(a[0], a[1], a[2], a[3]);
-  }
   static __device__ __forceinline__ void add(T& s, const T& x) {
     s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
   }
@@ -112,10 +101,6 @@ template <> struct SpmmVec<4> {
   static __device__ __forceinline__ T shfl_xor(const T& v, int d) {
     return make_float4(__shfl_xor_sync(0xffffffffu, v.x, d), __shfl_xor_sync(0xffffffffu, v.y, d),
                        __shfl_xor_sync(0xffffffffu, v.z, d), __shfl_xor_sync(0xffffffffu, v.w, d));
-  }
-  static __device__ __forceinline__ T shfl(const T& v, int src) {
-    return make_float4(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
-                       __shfl_sync(0xffffffffu, v.z, src), __shfl_sync(0xffffffffu, v.w, src));
   }
 };
 

@@ -27,7 +27,8 @@
 // busiest slice runs at 80 % of its peak).  With 32 warps of 14 gathers per lane there are
 // up to 14,336 gathers in flight per SM, twice the split kernel's; a warp instruction count
 // of 1.4 per nonzero instead of 2.4 (no atomics on shared memory, no zeroed sums, one pass
-// over the products) leaves the load path to them.  R-MAT scale 24, f32: 1.158 -> 0.928 ms.
+// over the products) leaves the load path to them.  R-MAT scale 24, f32: 1.158 -> 0.99 ms (0.93 to 1.03 on
+// other boxes).
 // f64: this GPU has two FP64 lanes per SM and clock, so a warp instruction of FP64 holds the
 // SM's pipe for 16 cycles; the fused multiply-add halves the work per nonzero (the split
 // kernel multiplies, stores and adds) and row ends cost one add instead of two atomics.
@@ -503,8 +504,8 @@ __global__ void __launch_bounds__(kWalkThreads, CTAS)
   if (tid == 0) g.red->arrive = 0u;
 }
 
-// Resident CTAs per SM: 32 warps for 4-byte sums (R-MAT scale 24: 0.929 ms, 24 warps 0.952,
-// 16 warps 1.012), 24 for 8-byte ones, whose buffers (5.8 KB a warp) would leave L1 too
+// Resident CTAs per SM: 32 warps for 4-byte sums (R-MAT scale 24, on one box: 0.929 ms, 24 warps
+// 0.952, 16 warps 1.012), 24 for 8-byte ones, whose buffers (5.3 KB a warp) would leave L1 too
 // little at 32 (R-MAT scale 22 with 30 % empty rows, with 46 KB a CTA: 0.216 ms; 32 warps 0.261, 16 warps 0.224).
 template <typename AT>
 constexpr int kWalkCtas = sizeof(AT) == 8 ? 3 : 4;

@@ -69,3 +69,25 @@ def test_tiles_of_a_long_row_add_up_in_64_bits(cuda_device, k, dtype):
     else:
         y = mb.spmm(p, vals, torch.ones(4, k, device="cuda"))
     assert (y == float(v.sum())).all()
+
+
+@pytest.mark.parametrize("k", [1, 8, 32])
+@pytest.mark.parametrize("what", ["inf", "both", "nan", "overflow"])
+def test_long_rows_that_are_not_finite(cuda_device, k, what):
+    """Rows of 20 tiles with an infinity, both, a NaN, or finite terms whose sum overflows."""
+    rows, length = 2000, 448 * 20
+    v = np.ones(length, np.float32)
+    at = 8 * 448
+    if what in ("inf", "both"):
+        v[at] = np.inf
+    if what == "both":
+        v[at + 2000] = -np.inf
+    if what == "nan":
+        v[at] = np.nan
+    if what == "overflow":
+        v[:] = 3e38 / 4000
+    row_ptr = torch.arange(0, rows * length + 1, length, dtype=torch.int32, device="cuda")
+    vals = torch.from_numpy(np.tile(v, rows)).cuda()
+    p = mb.plan(row_ptr, torch.zeros(rows * length, dtype=torch.int32, device="cuda"), rows, 4)
+    y = mb.spmv(p, vals, torch.ones(4, device="cuda")) if k == 1 else mb.spmm(p, vals, torch.ones(4, k, device="cuda"))
+    assert (torch.isnan(y) if what in ("both", "nan") else y == float("inf")).all()
