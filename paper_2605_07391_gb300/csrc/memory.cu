@@ -45,6 +45,13 @@ cudaMemPool_t pool_of(int dev) {
   return pool;
 }
 
+// A refused allocation is the caller's answer, not an error of the next launch: the runtime would
+// report it again there.
+cudaError_t answered(cudaError_t e) {
+  if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+  return e;
+}
+
 }  // namespace
 
 // The block may be used by work queued on `st` from here on, and by any stream once `st` has been
@@ -65,19 +72,18 @@ cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t st) {
     cudaStreamSynchronize(st);
     cudaMemPoolTrimTo(pool, 0);
   }
-  return cudaMalloc(p, bytes ? bytes : 1);
+  return answered(cudaMalloc(p, bytes ? bytes : 1));
 }
 
 cudaError_t dev_malloc(void** p, size_t bytes) {
-  const cudaError_t e = cudaMalloc(p, bytes);
+  const cudaError_t e = answered(cudaMalloc(p, bytes));
   if (e != cudaErrorMemoryAllocation) return e;
   int dev = 0;
   cudaGetDevice(&dev);
   const cudaMemPool_t pool = pool_of(dev);
   if (!pool) return e;
-  cudaGetLastError();
   cudaMemPoolTrimTo(pool, 0);
-  return cudaMalloc(p, bytes);
+  return answered(cudaMalloc(p, bytes));
 }
 
 cudaError_t device_wait(int device) {
@@ -88,7 +94,7 @@ cudaError_t device_wait(int device) {
   // stream of any thread is being captured: it fails and breaks the capture.
   const RelaxedCalls relaxed;
   void* block = nullptr;
-  cudaError_t e = cudaMalloc(&block, 256);
+  cudaError_t e = answered(cudaMalloc(&block, 256));
   e = e == cudaSuccess ? cudaFree(block) : cudaDeviceSynchronize();
   if (current != device) cudaSetDevice(current);
   return e;

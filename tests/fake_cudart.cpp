@@ -6,7 +6,8 @@
 //   * cudaDeviceSynchronize waits for the current device; while a stream is being captured it
 //     fails and breaks the capture;
 //   * cudaMalloc and cudaFree break a global-mode capture unless the thread is in relaxed mode;
-//   * idle memory of a pool counts against the device's memory until the pool is trimmed.
+//   * idle memory of a pool counts against the device's memory until the pool is trimmed;
+//   * a refused allocation is the next cudaGetLastError's answer too.
 #include <cuda_runtime.h>
 
 #include <cstdlib>
@@ -20,6 +21,7 @@ int g_dev = 0, g_busy[2] = {0, 0}, g_violations = 0, g_capturing = 0, g_broken =
 cudaStreamCaptureMode g_mode = cudaStreamCaptureModeGlobal;
 void* g_set = nullptr;      // the first range cleared since fake_reset
 size_t g_set_bytes = 0;
+cudaError_t g_last = cudaSuccess;
 size_t g_used = 0, g_idle = 0, g_limit = ~size_t(0) >> 1;
 
 cudaError_t unsafe_call() {
@@ -42,6 +44,7 @@ void fake_reset() {
   g_limit = ~size_t(0) >> 1;
   g_idle = 0;
   g_set = nullptr;
+  g_last = cudaSuccess;
 }
 void fake_busy(int dev, int busy) { g_busy[dev] = busy; }
 void fake_capture(int on) { g_capturing = on; }
@@ -54,6 +57,11 @@ void* fake_first_set(size_t* bytes) { *bytes = g_set_bytes; return g_set; }
 size_t fake_used() { return g_used; }
 size_t fake_idle() { return g_idle; }
 
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = g_last;
+  g_last = cudaSuccess;
+  return e;
+}
 cudaError_t cudaGetDevice(int* d) { *d = g_dev; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { g_dev = d; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() {
@@ -73,14 +81,14 @@ cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) {
 cudaError_t cudaMalloc(void** p, size_t n) {
   *p = nullptr;
   if (cudaError_t e = unsafe_call()) return e;
-  if (g_used + g_idle + n > g_limit) return cudaErrorMemoryAllocation;
+  if (g_used + g_idle + n > g_limit) return g_last = cudaErrorMemoryAllocation;
   ++g_mallocs;
   return take(p, n, false);
 }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
   *p = nullptr;
   const size_t reuse = n < g_idle ? n : g_idle;
-  if (g_used + g_idle + n - reuse > g_limit) return cudaErrorMemoryAllocation;
+  if (g_used + g_idle + n - reuse > g_limit) return g_last = cudaErrorMemoryAllocation;
   g_idle -= reuse;
   return take(p, n, true);
 }

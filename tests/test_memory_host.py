@@ -101,3 +101,29 @@ def test_first_spmm_of_a_plan_takes_pool_memory(lib, k):
     assert lib.fake_mallocs() == before
     assert (lib.fake_used() == used) == (k == 1)      # one column needs no accumulators
     lib.merbit_plan_destroy(h)
+
+
+@pytest.mark.parametrize("call", ["plan", "transpose", "batch", "autotune", "bicgstab"])
+def test_a_refused_allocation_is_reported_once(lib, call):
+    lib.fake_reset()
+    m = fr.Pattern(lib)
+    h = m.plan()
+    v, x, y = (np.zeros(s + 2) for s in (m.nnz, m.n, m.n))
+    vp, out = ctypes.c_void_p, ctypes.c_void_p()
+    at = [vp(t.ctypes.data + -t.ctypes.data % 16) for t in (v, x, y)]
+    lib.fake_limit(100)
+    if call == "plan":
+        st = lib.merbit_plan_ex(*m.args(), 14, 8, None, ctypes.byref(out))
+    elif call == "transpose":
+        st = lib.merbit_transpose(*m.args(), None, ctypes.byref(out))
+    elif call == "batch":
+        off, (rp, col, n, _, nnz) = np.array([0, m.n], np.int64), m.args()
+        st = lib.merbit_batch_plan(rp, col, n, nnz, vp(off.ctypes.data), 1, 14, None, ctypes.byref(out))
+    elif call == "autotune":
+        cand, best = (ctypes.c_int * 1)(14), ctypes.c_int()
+        st = lib.merbit_autotune_sigma(*m.args(), 1, at[0], cand, 1, 1, None, ctypes.byref(best), None)
+    else:
+        st = lib.merbit_bicgstab(h, *at, ctypes.c_double(0.0), 2, None, None, None, None, None)
+    assert st == 3, lib.merbit_last_error()      # ENOMEM
+    assert lib.merbit_spmv_ex(h, 1, 1, *at, 0, None) == 0, lib.merbit_last_error()
+    lib.merbit_plan_destroy(h)
