@@ -533,7 +533,7 @@ inline int walk_unit(int64_t tiles, int64_t warps, int W) {
 
 // Products of at most this many unit boundaries are finished by the kernel's last CTA: a launch less,
 // but one CTA for all of them.  R-MAT-like graphs, refinement to 1e-10 with this limit at 1,024 and
-// at 2,048: 1,237 tiles 2.27 and 2.10 ms, 1,439 tiles 2.69 and 2.55, 1,718 and 1,897 tiles level;
+// at 2,048: 1,237 tiles 2.27 and 2.10 ms, 1,369 tiles 2.69 and 2.55, 1,718 and 1,897 tiles level;
 // BiCGSTAB, an iteration: 1,499 tiles 59.2 and 59.9 us.
 constexpr int64_t kWalkFoldMax = 1440;
 
