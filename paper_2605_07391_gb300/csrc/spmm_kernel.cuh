@@ -104,12 +104,12 @@ template <> struct SpmmVec<4> {
   }
 };
 
-// Y[r, c..c+VW) = sum.  YVEC: the slices of Y are 16-byte aligned and kc is a multiple
+// Y[r, c..c+VW) = (scale *) sum.  YVEC: the slices of Y are 16-byte aligned and kc is a multiple
 // of VW; otherwise single columns below kc are stored.
 struct SpmmOut {
   float* y;
   int64_t ldy;
-  float scale;     // of the values (SCALED)
+  float scale;
   int kc;          // columns of the chunk
   bool gated;      // the launch does nothing once an iterative driver has set the stop flag
   __device__ __forceinline__ bool skip(const RedState* red) const {
@@ -117,24 +117,31 @@ struct SpmmOut {
   }
 };
 
+template <bool SCALED>
+__device__ __forceinline__ float spmm_scaled(float v, float scale) {
+  if constexpr (SCALED) return scale * v;
+  else return v;
+}
+
 // Predicated stores of a slice (no branch: lanes of a warp end rows at different steps; no memory
 // clobber: nothing in the kernel reads Y, and loads may move over them).
-template <int VW, bool YVEC>
-__device__ __forceinline__ void spmm_store_if(uint32_t pred, float* p, const typename SpmmVec<VW>::T& v,
+template <int VW, bool YVEC, bool SCALED>
+__device__ __forceinline__ void spmm_store_if(uint32_t pred, float* p, const typename SpmmVec<VW>::T& v, float scale,
                                               int left) {
   using V = SpmmVec<VW>;
   if constexpr (YVEC && VW == 4) {
     asm volatile(
         "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t"
         "@q st.global.v4.f32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(pred),
-        "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
+        "l"(p), "f"(spmm_scaled<SCALED>(v.x, scale)), "f"(spmm_scaled<SCALED>(v.y, scale)),
+        "f"(spmm_scaled<SCALED>(v.z, scale)), "f"(spmm_scaled<SCALED>(v.w, scale)));
   } else {
 #pragma unroll
     for (int i = 0; i < VW; ++i)
       asm volatile(
           "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t"
           "@q st.global.f32 [%1], %2;\n\t}" ::"r"(i < left ? pred : 0u),
-          "l"(p + i), "f"(V::get(v, i)));
+          "l"(p + i), "f"(spmm_scaled<SCALED>(V::get(v, i), scale)));
   }
 }
 
@@ -213,12 +220,6 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
     else
       return reinterpret_cast<const float*>(reinterpret_cast<const char*>(Xc) +
                                             (uint64_t)(uint32_t)col * ((uint32_t)ldx * 4u));
-  };
-  // the scale goes to the values, one a nonzero: to the sums it would be VW products a step, stored or
-  // not (personalised PageRank, 2^22 vertices, k = 32: 1.33 ms an update, 1.23)
-  auto weight = [&](float v) {
-    if constexpr (SCALED) return out.scale * v;
-    else return v;
   };
   auto y_row = [&](int r) { return out.y + c + (int64_t)r * out.ldy; };
   auto unit_start = [&](int r) {
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
         VT part = V::zero();
 #pragma unroll
         for (int u = 0; u < U1; ++u)
-          if (b0 + u * L < ntile) V::fma(weight(sv[pad + b0 + u * L]), xv[u], part);
+          if (b0 + u * L < ntile) V::fma(sv[pad + b0 + u * L], xv[u], part);
         V::add(sum, part);
       }
       columns_read();
@@ -363,10 +364,10 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
         asm volatile("" : "+r"(rw), "+r"(dw));
 #pragma unroll
         for (int k = 0; k < KS; ++k) {
-          const float w = weight(vp[k]);
+          const float w = vp[k];
           if ((rw >> k) & 1u) V::fma(w, xv[k], sum);
           V::store_shared_if(first & (1u << k), s_head, sum);
-          spmm_store_if<VW, YVEC>((dw ^ first) & c_ok & (1u << k), yp, sum, left);
+          spmm_store_if<VW, YVEC, SCALED>((dw ^ first) & c_ok & (1u << k), yp, sum, out.scale, left);
           if ((dw >> k) & 1u) {
             sum = V::zero();
             yp += out.ldy;
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
           if (y0 == y_unit) {
             if (c_ok) add_acc(t_start, in, V::zero());
           } else {
-            spmm_store_if<VW, YVEC>(c_ok, y_row(y0), in, left);
+            spmm_store_if<VW, YVEC, SCALED>(c_ok, y_row(y0), in, out.scale, left);
           }
         }
         __syncwarp();
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CTAS)
   }
 }
 
-// Rows of the unit boundaries: Y[r, c] = acc[set][c], accumulator cleared.  Every
+// Rows of the unit boundaries: Y[r, c] = scale * acc[set][c], accumulator cleared.  Every
 // distinct row is written once, by its first boundary.
 template <int KC>
 __global__ void __launch_bounds__(256) merbit_spmm_finalize_kernel(const Geometry g, double* __restrict__ acc,
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(256) merbit_spmm_finalize_kernel(const Geometr
     double* a = acc + p;
     const double tot = *a;
     *a = 0.0;
-    out.y[(int64_t)r * out.ldy + cc] = static_cast<float>(tot);
+    out.y[(int64_t)r * out.ldy + cc] = static_cast<float>(static_cast<double>(out.scale) * tot);
   }
 }
 
